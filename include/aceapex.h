@@ -107,13 +107,12 @@ typedef struct {
                              before it is left to the later, barrier-separated rounds; 0xFFFFFFFF = no limit
                              short of timeout_us (pieces are handed out in output order, so the lowest
                              unfinished one always has final sources and the first round finishes them all);
-                             0 = automatic: no limit while the pending pieces are at most 16 per thread of the
-                             pass's grid and 256 per block, else 4000 (many pieces with long chains would clog
-                             the hand-out), or, for an archive with level bodies, level order with 20000 */
-    uint32_t ignore_levels; /* 0: a whole-archive decode of an archive with level bodies (flags bit1) takes
-                               the cross-block matches level by level (paper, "Depth Does Not Govern
-                               Latency": one round per wave, every piece attempted once, a piece whose
-                               hint proves too low left to the later rounds); 1: ignore the level bodies */
+                             0 = automatic: output order, no limit; any other value takes the pieces of
+                             an archive with level bodies in level order (see ignore_levels) */
+    uint32_t ignore_levels; /* 0: with wait_ns set, a whole-archive decode of an archive with level bodies
+                               (flags bit1) takes the cross-block matches level by level (paper, "Depth Does
+                               Not Govern Latency": the waves; a piece whose hint proves too low is left to
+                               the later rounds); 1: ignore the level bodies */
 } aceapex_dec_params;
 
 /* Timing of the last call, measured with CUDA events on the call's stream

@@ -278,8 +278,9 @@ static int enqueue_decode(aceapex_ctx* c, aceapex_archive* A, const void* d_arc,
     job.lists[0] = (JobDev::ListEnt*)c->lists.p;
     job.lists[1] = (JobDev::ListEnt*)c->lists.p + std::max<uint64_t>(P.span_slots, 1);
     if (hi <= lo) return ACEAPEX_OK;
-    if ((P.flags & kFlagLevels) && !c->params.ignore_levels && c->params.variant != ACEAPEX_VARIANT_PLAIN) {
-        // level-ordered cross-block rounds: one row of the level table per block
+    if ((P.flags & kFlagLevels) && !c->params.ignore_levels && c->params.wait_ns != 0 &&
+        c->params.variant != ACEAPEX_VARIANT_PLAIN) {
+        // level-ordered cross-block pass: one row of the level table per block
         const uint32_t Lg = std::max<uint32_t>(1, std::min<uint32_t>(P.max_level, kMaxLevel));
         if ((e = c->lvl_tab.ensure(nb * (Lg + 1) * 4)) != cudaSuccess) return cuda_fail(c, e, "level-table allocation");
         if ((e = c->lvl_off.ensure((nb * Lg + 2 * Lg + 1) * 4)) != cudaSuccess)
@@ -290,7 +291,6 @@ static int enqueue_decode(aceapex_ctx* c, aceapex_archive* A, const void* d_arc,
         job.lvl_off = (uint32_t*)c->lvl_off.p;
         job.lvl_list = (JobDev::ListEnt*)c->lvl_list.p;
         job.lvl_cap = (uint32_t)std::max<uint64_t>(P.span_slots, 1);
-        job.lvl_min_pieces = lvl_auto_min_pieces(c);
         job.n_levels = Lg;
         job.flags |= kJobLevels;
     }

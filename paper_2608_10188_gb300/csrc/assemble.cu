@@ -21,14 +21,14 @@
 //     chain leaves the block become pending spans.
 //   * the block is written with coalesced 16-byte stores; its pending-byte
 //     bitmap and pending spans go beside it.
-// k_external (warps take blocks in ascending order, one lane per span):
+// k_external (warps take parts of blocks in ascending order, one lane per span):
 //   after the kernel boundary every literal and every in-block match byte is
 //   final, so a pending span waits only on the spans its source really
 //   depends on, which lie at lower positions and were taken earlier: the
-//   ascending order makes the bounded waits deadlock-free.  Spans that wait
-//   too long (many pieces, long chains) go to work lists, staged per warp in
-//   shared memory; barrier-separated rounds walk the lists until they are
-//   empty, each round finishing at least the lowest span.
+//   ascending order makes the bounded waits deadlock-free.  Under an explicit
+//   wait limit (wait_ns), spans that wait for longer go to work lists, staged
+//   per warp in shared memory; barrier-separated rounds walk the lists until
+//   they are empty, each round finishing at least the lowest span.
 #include <algorithm>
 
 #include <mutex>
@@ -44,152 +44,193 @@ __global__ void __launch_bounds__(kLocThreads, 6) k_local(JobDev job) {
 }
 
 // ---- cross-block pass --------------------------------------------------------------------
-// Are the bytes [s, e) (absolute) final?  The local pass writes every
-// block's pending-byte bitmap; a clear bit means a final byte.  The loads are
-// acquire loads: a lane that sees its piece's source bits clear is ordered
-// after the release that cleared them, and the warp barrier before the copy
-// carries that order to the lanes that read the bytes (no fence per attempt).
-// A range of at most 32 bytes (every piece) covers at most two bitmap words,
-// possibly of two blocks: both are loaded before either is tested.
-__device__ __forceinline__ bool src_final(const ArcJob& L, uint64_t s, uint64_t e) {
-    if (e - s <= 32) {
-        const uint64_t l = e - 1;
-        const uint64_t s0 = slot_of(L, s >> 14), s1 = slot_of(L, l >> 14);
-        if (s0 == kNoSlot || s1 == kNoSlot) return false;  // not in this decode's output: never final
-        const uint32_t o0 = (uint32_t)(s & (kBlock - 1)), o1 = (uint32_t)(l & (kBlock - 1));
-        const uint32_t* p0 = L.pmap + s0 * (kBlock / 32) + (o0 >> 5);
-        const uint32_t* p1 = L.pmap + s1 * (kBlock / 32) + (o1 >> 5);
-        const uint32_t lo0 = 0xffffffffu << (o0 & 31);         // bits from o0 on in its word
-        const uint32_t hi1 = 0xffffffffu >> (31 - (o1 & 31));  // bits up to o1 in its word
-        if (p0 == p1) return (ld_acquire_u32(p0) & lo0 & hi1) == 0;
-        const uint32_t w0 = ld_acquire_u32(p0), w1 = ld_acquire_u32(p1);
-        return ((w0 & lo0) | (w1 & hi1)) == 0;
-    }
-    for (uint64_t a = s >> 14; a <= (e - 1) >> 14; a++) {
-        const uint64_t A = a << 14;
-        const uint32_t lo = (uint32_t)((s > A ? s : A) - A);
-        const uint32_t hi = (uint32_t)((e < A + kBlock ? e : A + kBlock) - A);
-        const uint64_t sl = slot_of(L, a);
-        if (sl == kNoSlot) return false;
-        const uint32_t* pm = L.pmap + sl * (kBlock / 32);
-        for (uint32_t w = lo >> 5; w <= ((hi - 1) >> 5); w++)
-            if (ld_acquire_u32(pm + w) & range_mask(w, lo, hi)) return false;  // pairs with the released clears
-    }
-    return true;
+// What the pass needs of the archive that a piece belongs to.  A job over one
+// archive keeps it in the kernel's parameters; in a batch each lane holds its
+// own piece's.
+struct ArcView {
+    uint8_t* out;
+    uint32_t* pmap;
+    const uint32_t* slot;
+    uint64_t total;
+};
+__device__ __forceinline__ ArcView view_of(const ArcJob& J) { return ArcView{J.out, J.pmap, J.slot, J.total}; }
+__device__ __forceinline__ uint64_t slot_of(const ArcView& V, uint64_t a) { return V.slot ? V.slot[a] : a; }
+__device__ __forceinline__ uint64_t out_off(const ArcView& V, uint64_t pos) {
+    return V.slot ? (uint64_t)V.slot[pos >> 14] * kBlock + (pos & (kBlock - 1)) : pos;
 }
 
-constexpr int kExtThreads = 1024;  // one CTA per SM: grid barriers stay cheap
-constexpr uint32_t kRound0WaitNs = 4000;  // wait of a round-0 piece for its sources when they are many
-constexpr uint32_t kWaitAllPerLane = 16;   // pieces per grid lane up to which round 0 waits without limit,
-constexpr uint32_t kWaitAllPerItem = 256;  // ... and per block: a warp holding a block's pieces on long chains
-                                           // would stall its hand-out
-constexpr uint32_t kLevelWaitNs = 20000;   // wait of a piece handed out in level order
+// Are the bytes [s, e) (absolute, at most 32 of them) final?  The local pass
+// writes every block's pending-byte bitmap; a clear bit means a final byte.
+// The loads are acquire loads: a lane that sees its piece's source bits clear
+// is ordered after the release that cleared them, and the warp barrier before
+// a copy by other lanes carries that order to them (no fence per attempt).
+// At most two bitmap words, possibly of two blocks: both are loaded before
+// either is tested.
+__device__ __forceinline__ bool src_final(const ArcView& V, uint64_t s, uint64_t e) {
+    const uint64_t l = e - 1;
+    const uint64_t s0 = slot_of(V, s >> 14), s1 = slot_of(V, l >> 14);
+    if (s0 == kNoSlot || s1 == kNoSlot) return false;  // not in this decode's output: never final
+    const uint32_t o0 = (uint32_t)(s & (kBlock - 1)), o1 = (uint32_t)(l & (kBlock - 1));
+    const uint32_t* p0 = V.pmap + s0 * (kBlock / 32) + (o0 >> 5);
+    const uint32_t* p1 = V.pmap + s1 * (kBlock / 32) + (o1 >> 5);
+    const uint32_t lo0 = 0xffffffffu << (o0 & 31);         // bits from o0 on in its word
+    const uint32_t hi1 = 0xffffffffu >> (31 - (o1 & 31));  // bits up to o1 in its word
+    if (p0 == p1) return (ld_acquire_u32(p0) & lo0 & hi1) == 0;
+    const uint32_t w0 = ld_acquire_u32(p0), w1 = ld_acquire_u32(p1);
+    return ((w0 & lo0) | (w1 & hi1)) == 0;
+}
+
+// One CTA per SM: grid barriers stay cheap, and more warps are no faster (768 x 2
+// and 1024 x 2 threads per SM: 1178 and 1338 us on 11 M text pieces, against
+// 1108): the pass is bound by the memory system's latency under load.
+constexpr int kExtThreads = 1024;
+// Pieces a hand-out ticket of round 0 covers, about: a block's pieces are cut
+// into as many equal parts as that takes on average over the job.  Handed out
+// by whole blocks, a text block's 900 pieces run on one warp, a small file
+// leaves most warps without work, and a large one has all of its blocks in
+// flight at once, so that chains between them clog the lanes; in parts, the
+// pieces in flight are a narrow window of the output, and a wait without limit
+// pays at every size.  Zipf text: 1 MiB 195 -> 35 us, 4 MiB 238 -> 55, 16 MiB
+// 242 -> 82, 64 MiB 418 -> 297, 200 MiB 1091 (in level order) -> 760; DNA-like
+// 4 MiB 43 -> 34, 64 MiB 70 -> 59.  With parts of 32 / 128 pieces the 200 MiB text takes
+// 881 / 832 us, and DNA-like 64 MiB 61 / 72.
+constexpr uint32_t kPartPieces = 64;
 
 // Are the bytes a piece reads final?  (period 0: [src, src+len); otherwise the
 // residues phase.. of the period window [src, src+period), one or two ranges.)
-__device__ __forceinline__ bool piece_final(const ArcJob& L, uint64_t src, uint32_t phase, uint32_t period,
+__device__ __forceinline__ bool piece_final(const ArcView& V, uint64_t src, uint32_t phase, uint32_t period,
                                             uint32_t len) {
-    if (period == 0) return src_final(L, src, src + len);
-    if (len >= period) return src_final(L, src, src + period);
-    if (phase + len <= period) return src_final(L, src + phase, src + phase + len);
-    return src_final(L, src + phase, src + period) && src_final(L, src, src + (phase + len - period));
+    uint32_t lo = 0, hi = len, wrap = 0;  // [src + lo, src + hi), then [src, src + wrap)
+    if (period) {
+        lo = len >= period ? 0 : phase;
+        hi = len >= period ? period : min(phase + len, period);
+        wrap = len >= period || phase + len <= period ? 0 : phase + len - period;
+    }
+    return src_final(V, src + lo, src + hi) && (wrap == 0 || src_final(V, src, src + wrap));
 }
 
-constexpr int kCopyBatch = 8;
-constexpr int kPlainBatch = 8;  // loads in flight before their stores, published-address copies (16: no faster)
+constexpr int kSlowBatch = 4;  // byte-copied pieces whose loads are in flight together
+
+// Copy len <= 32 bytes from sa to da, any alignments, by one lane: the aligned
+// 16-byte words that hold the source bytes (three at most), a barrel shift to
+// the destination's 8-byte words, whole words as 8-byte stores, and the ragged
+// ends as a 1-, a 2- and a 4-byte store each, as far as they need them.  Only
+// words that hold a source byte are read, only the len bytes are written.  (A
+// warp's 32 pieces take about 600 instructions in all; moved a byte per lane,
+// a piece at a time, they took 1,340, and the output-order pass over 64 MiB of
+// text 474 us instead of 426.)
+__device__ __forceinline__ void copy_piece(const uint8_t* sa, uint8_t* da, uint32_t len) {
+    const uint32_t off = (uint32_t)(uintptr_t)sa & 15, d0 = (uint32_t)(uintptr_t)da & 7, E = d0 + len;
+    const uint4* S = reinterpret_cast<const uint4*>(sa - off);
+    const uint4 z = make_uint4(0, 0, 0, 0);
+    const uint4 a = __ldcg(S), b = off + len > 16 ? __ldcg(S + 1) : z, c = off + len > 32 ? __ldcg(S + 2) : z;
+    // w: the source from 8 bytes before S; the destination's word 0 starts at
+    // byte e of it
+    uint32_t w[18] = {0, 0, a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w, 0, 0, 0, 0};
+    const uint32_t e = off + 8 - d0, q = e >> 2, sh = 8 * (e & 3);
+#pragma unroll
+    for (int i = 0; i < 14; i++) w[i] = q & 4 ? w[i + 4] : w[i];
+#pragma unroll
+    for (int i = 0; i < 12; i++) w[i] = q & 2 ? w[i + 2] : w[i];
+#pragma unroll
+    for (int i = 0; i < 11; i++) w[i] = q & 1 ? w[i + 1] : w[i];
+#pragma unroll
+    for (int i = 0; i < 10; i++) w[i] = __funnelshift_r(w[i], w[i + 1], sh);
+    uint8_t* D = da - d0;
+    uint32_t p = d0;  // up to the next 8-byte boundary
+    if ((p & 1) && p + 1 <= E) {
+        D[p] = (uint8_t)((p & 4 ? w[1] : w[0]) >> (8 * (p & 3)));
+        p += 1;
+    }
+    if ((p & 2) && p + 2 <= E) {
+        *reinterpret_cast<uint16_t*>(D + p) = (uint16_t)((p & 4 ? w[1] : w[0]) >> (8 * (p & 3)));
+        p += 2;
+    }
+    if ((p & 4) && p + 4 <= E) {
+        *reinterpret_cast<uint32_t*>(D + p) = w[1];
+        p += 4;
+    }
+    uint32_t t0 = w[0], t1 = w[1];  // the word that holds byte p
+#pragma unroll
+    for (int k = 0; k < 5; k++) {
+        if (p >= 8u * k) {
+            t0 = w[2 * k];
+            t1 = w[2 * k + 1];
+        }
+        if (p == 8u * k && p + 8 <= E) {
+            *reinterpret_cast<uint2*>(D + 8 * k) = make_uint2(t0, t1);
+            p += 8;
+        }
+    }
+    if (p + 4 <= E) {
+        *reinterpret_cast<uint32_t*>(D + p) = t0;
+        p += 4;
+    }
+    if (p + 2 <= E) {
+        *reinterpret_cast<uint16_t*>(D + p) = (uint16_t)((p & 4 ? t1 : t0) >> (8 * (p & 3)));
+        p += 2;
+    }
+    if (p < E) D[p] = (uint8_t)((p & 4 ? t1 : t0) >> (8 * (p & 3)));
+}
+
 // A warp's attempt at its lanes' pieces (lane `has` a piece `rec` of the
-// block in output slot `dslot`, all of archive L).  Each lane checks its own
-// piece; the ready pieces are then copied by the whole warp, lane i moving
-// byte i (one coalesced request per piece), eight pieces' loads in flight
-// before their stores (in a whole-archive job from addresses that the
-// pieces' owners publish); after one fence (the release) the owners clear
-// the pieces' pending bits with relaxed atomic ANDs.  Returns true on the
-// lanes whose piece is done.
-__device__ bool try_pieces(bool has, const ArcJob& L, uint32_t dslot, SpanRec rec, SpanRec* wrec, uint64_t* wdst,
-                           int lane) {
+// block in output slot `dslot`, of archive L).  Each lane checks its own
+// piece and copies it when it is ready; after one fence (the release) the
+// lanes clear the pieces' pending bits with relaxed atomic ANDs.  Returns true
+// on the lanes whose piece is done.
+//
+// Periodic pieces, pieces whose last 16-byte source word would end beyond the
+// output and, in jobs with slots, pieces whose source crosses a block boundary
+// go by bytes: their owners publish them in shared memory and the warp walks
+// them, lane i moving byte i.
+__device__ __forceinline__ bool try_pieces(bool has, const ArcView& L, uint32_t dslot, SpanRec rec, SpanRec* wrec,
+                                           uint64_t* wdst, int lane) {
     const uint64_t src = (uint64_t)rec.x | ((uint64_t)(rec.y & 0xff) << 32);
     const uint32_t phase = (rec.y >> 8) & 0xffff, period = rec.w, o = rec.z & 0xffff, len = rec.z >> 16;
     const bool ready = has && piece_final(L, src, phase, period, len);
     const uint32_t rmask = __ballot_sync(ACX_FULL, ready);
     if (!rmask) return false;
     uint8_t* g = L.out;
-    uint32_t m = rmask;
-    if (!L.slot) {
-        // a whole-archive job (blocks at their own offsets): each ready lane
-        // publishes its piece's source and destination addresses, length and
-        // period in the slot of its rank among the ready lanes, and the warp
-        // walks the slots in order
-        const uint8_t** wsa = reinterpret_cast<const uint8_t**>(wrec);  // [rank]: source address
-        uint8_t** wda = reinterpret_cast<uint8_t**>(wrec) + 32;         // [rank]: destination address
-        uint32_t* wln = reinterpret_cast<uint32_t*>(wdst);              // [rank]: length | phase << 8
-        uint32_t* wpp = wln + 32;                                        // [rank]: period | M << 16
-        if (ready) {
-            const uint32_t r = __popc(rmask & ((1u << lane) - 1));
-            wsa[r] = g + src;
-            wda[r] = g + (uint64_t)dslot * kBlock + o;
+    uint8_t* dst = g + (uint64_t)dslot * kBlock + o;
+    const bool words = ready && period == 0 && (L.slot ? (src >> 14) == ((src + len - 1) >> 14)
+                                                      : ((src + len + 15) & ~15ull) <= L.total);
+    if (words) copy_piece(g + out_off(L, src), dst, len);
+    const uint32_t smask = __ballot_sync(ACX_FULL, ready && !words);
+    if (smask) {
+        uint64_t* wsa = reinterpret_cast<uint64_t*>(wrec);       // [rank]: source address (jobs with slots: position)
+        uint64_t* wda = reinterpret_cast<uint64_t*>(wrec) + 32;  // [rank]: destination address
+        uint32_t* wln = reinterpret_cast<uint32_t*>(wdst);       // [rank]: length | phase << 8
+        uint32_t* wpp = wln + 32;                                 // [rank]: period | M << 16
+        if (ready && !words) {
+            const uint32_t r = __popc(smask & ((1u << lane) - 1));
+            wsa[r] = L.slot ? src : (uint64_t)(g + src);
+            wda[r] = (uint64_t)dst;
             wln[r] = len | phase << 8;
             // a period below 32 takes the residue by a multiply-shift: for
             // x < 64, (x * ceil(2048 / p)) >> 11 is floor(x / p)
             wpp[r] = period | (period && period < 32 ? ((2047 + period) / period) << 16 : 0u);
         }
         __syncwarp();
-        const uint32_t nr = __popc(rmask);
-        // the walk is branch-free: predicated loads and stores, selects for
-        // the residue of a periodic piece (byte k reads (phase + k) mod period;
-        // phase < period, so with a period of 32 or more one subtraction does)
-        for (uint32_t b0 = 0; b0 < nr; b0 += kPlainBatch) {
-            uint32_t v[kPlainBatch / 4];
+        const uint32_t ns = __popc(smask);
+        // byte k of a periodic piece reads (phase + k) mod period of its window
+        // (phase < period, so with a period of 32 or more one subtraction does)
+        for (uint32_t b0 = 0; b0 < ns; b0 += kSlowBatch) {
+            uint32_t v = 0;
+            bool mine[kSlowBatch];
 #pragma unroll
-            for (int u = 0; u < kPlainBatch / 4; u++) v[u] = 0;
-            uint32_t mine = 0;  // bit u: this lane moves a byte of piece b0 + u
-#pragma unroll
-            for (int u = 0; u < kPlainBatch; u++) {
+            for (int u = 0; u < kSlowBatch; u++) {
                 const uint32_t i = (b0 + u) & 31;
                 const uint32_t a = wln[i], pp = wpp[i];
                 const uint32_t per = pp & 0xffff, M = pp >> 16, x = (uint32_t)lane + (a >> 8);
                 const uint32_t k = M ? x - per * ((x * M) >> 11) : (per && x >= per ? x - per : x);
-                const bool p = b0 + u < nr && (uint32_t)lane < (a & 0xff);
-                const uint32_t b = p ? (uint32_t)__ldcg(wsa[i] + k) : 0u;
-                v[u >> 2] |= b << (8 * (u & 3));
-                mine |= (uint32_t)p << u;
+                mine[u] = b0 + u < ns && (uint32_t)lane < (a & 0xff);
+                const uint64_t q = wsa[i] + k;
+                if (mine[u])
+                    v |= (uint32_t)__ldcg(L.slot ? g + out_off(L, q) : reinterpret_cast<const uint8_t*>(q)) << (8 * u);
             }
 #pragma unroll
-            for (int u = 0; u < kPlainBatch; u++)
-                if (mine >> u & 1) wda[(b0 + u) & 31][lane] = (uint8_t)(v[u >> 2] >> (8 * (u & 3)));
-        }
-    } else {
-        wrec[lane] = rec;
-        wdst[lane] = (uint64_t)dslot * kBlock + o;
-        __syncwarp();
-        while (m) {
-            int ls[kCopyBatch];
-#pragma unroll
-            for (int u = 0; u < kCopyBatch; u++) {
-                ls[u] = m ? __ffs(m) - 1 : -1;
-                if (m) m &= m - 1;
-            }
-            uint32_t v[(kCopyBatch + 3) / 4];
-#pragma unroll
-            for (int u = 0; u < (kCopyBatch + 3) / 4; u++) v[u] = 0;
-#pragma unroll
-            for (int u = 0; u < kCopyBatch; u++) {
-                if (ls[u] >= 0) {
-                    const SpanRec r = wrec[ls[u]];
-                    if ((uint32_t)lane < (r.z >> 16)) {
-                        const uint64_t rs = (uint64_t)r.x | ((uint64_t)(r.y & 0xff) << 32);
-                        const uint32_t rp = r.w;
-                        const uint64_t q = rp ? rs + (((r.y >> 8) & 0xffff) + (uint32_t)lane) % rp : rs + lane;
-                        v[u >> 2] |= (uint32_t)__ldcg(g + out_off(L, q)) << (8 * (u & 3));
-                    }
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kCopyBatch; u++) {
-                if (ls[u] >= 0) {
-                    const uint32_t rl = wrec[ls[u]].z >> 16;
-                    if ((uint32_t)lane < rl) g[wdst[ls[u]] + lane] = (uint8_t)(v[u >> 2] >> (8 * (u & 3)));
-                }
-            }
+            for (int u = 0; u < kSlowBatch; u++)
+                if (mine[u]) reinterpret_cast<uint8_t*>(wda[(b0 + u) & 31])[lane] = (uint8_t)(v >> (8 * u));
         }
     }
     // release: every lane's stores (to other lanes' pieces too) happen before
@@ -278,9 +319,9 @@ __device__ void report_stalled(const JobDev& job, uint32_t in, uint32_t n, uint3
     }
 }
 
-// One pass over a list of n pieces (a work list, or a level's segment of the
-// level list) by warps w0, w0 + nw, ...: every piece is attempted once; the
-// unfinished ones go to work list `out`.
+// One pass over a list of n pieces by warps w0, w0 + nw, ...: every piece is
+// attempted once; the unfinished ones go to work list `out`.
+template <bool kMulti>
 __device__ void round_pass(const JobDev& job, const ListEnt* src, uint32_t out, uint32_t n, uint32_t w0, uint32_t nw,
                            SpanRec* wrec, uint64_t* wdst, ListEnt* sbuf, int lane) {
     uint32_t sn = 0;
@@ -289,20 +330,11 @@ __device__ void round_pass(const JobDev& job, const ListEnt* src, uint32_t out, 
         const bool has = i < n;
         ListEnt e{0, 0};
         if (has) e = src[i];
-        // (the lanes' pieces may come from several archives: one archive at a time)
-        const int arc_i = has ? find_arc(job, e.y) : -1;
-        bool done = false;
-        uint32_t todo = __ballot_sync(ACX_FULL, has);
-        while (todo) {
-            const int a0 = __shfl_sync(ACX_FULL, arc_i, __ffs(todo) - 1);
-            const bool mine = has && arc_i == a0;
-            const ArcJob J = load_arc(job, a0);
-            SpanRec r{0, 0, 0, 0};
-            if (mine) r = J.spans[e.x];
-            const bool d2 = try_pieces(mine, J, mine ? item_ref(J, e.y - J.item_base).slot : 0, r, wrec, wdst, lane);
-            if (mine) done = d2;
-            todo &= ~__ballot_sync(ACX_FULL, mine);
-        }
+        const ArcJob& J = kMulti ? job.arcs[has ? find_arc(job, e.y) : 0] : job.one;
+        SpanRec r{0, 0, 0, 0};
+        if (has) r = J.spans[e.x];
+        const uint32_t slot = has ? item_ref(J, e.y - J.item_base).slot : 0;
+        const bool done = try_pieces(has, view_of(J), slot, r, wrec, wdst, lane);
         append(has && !done, e, sbuf, sn, job.lists[out], &job.counters[kListCnt + out], lane);
     }
     stage_flush(sbuf, sn, job.lists[out], &job.counters[kListCnt + out], lane);
@@ -312,13 +344,14 @@ __device__ void round_pass(const JobDev& job, const ListEnt* src, uint32_t out, 
 // entries and the count of the other list is zero.  Rounds are separated by
 // CTA barriers; the same progress argument as the grid rounds ends them.
 constexpr uint32_t kSoloMax = 4 * kExtThreads;  // lists up to four CTA-wide passes
+template <bool kMulti>
 __device__ void solo_rounds(const JobDev& job, uint32_t in, uint32_t n, uint32_t round, uint64_t deadline,
                             SpanRec* wrec, uint64_t* wdst, ListEnt* sbuf, int lane) {
     __shared__ uint32_t n_next;
     const uint32_t warp = threadIdx.x >> 5, nw = kExtThreads / 32;
     for (;;) {
         const uint32_t out = in ^ 1u;
-        round_pass(job, job.lists[in], out, n, warp, nw, wrec, wdst, sbuf, lane);
+        round_pass<kMulti>(job, job.lists[in], out, n, warp, nw, wrec, wdst, sbuf, lane);
         __syncthreads();  // every append of this round is visible to the CTA
         if (threadIdx.x == 0) {
             n_next = *((volatile uint32_t*)&job.counters[kListCnt + out]);
@@ -354,22 +387,6 @@ __device__ void solo_rounds(const JobDev& job, uint32_t in, uint32_t n, uint32_t
 //     level-l piece in output order (k_level_fill: one warp per item, reading
 //     each piece's level from its record).
 constexpr int kScanThreads = 1024;
-// Does the cross-block pass hand pieces out in level order?  Only in jobs
-// with level tables, and under the automatic policy only when pieces are
-// many per lane of the pass: with few, output order with waits that last as
-// long as needed resolves the chains at the latency of one copy per level and
-// needs no list.  Every kernel after the local pass reads the same final
-// count, so they all decide alike.
-__device__ __forceinline__ bool few_pieces(const JobDev& job, uint64_t lanes) {
-    const uint64_t pieces = *((volatile const uint32_t*)&job.counters[kStatPending]);
-    return pieces <= kWaitAllPerLane * lanes && pieces <= (uint64_t)kWaitAllPerItem * job.n_items;
-}
-__device__ __forceinline__ bool use_level_order(const JobDev& job) {
-    if (!job.lvl_tab) return false;
-    if (job.wait_ns != 0) return true;
-    return !few_pieces(job, job.lvl_min_pieces / kWaitAllPerLane);
-}
-
 // A decode whose local pass timed out left blocks unprocessed, so their level
 // rows, piece counts and records may be stale: the passes after it do nothing.
 __device__ __forceinline__ bool local_pass_timed_out(const JobDev& job) {
@@ -378,7 +395,7 @@ __device__ __forceinline__ bool local_pass_timed_out(const JobDev& job) {
 
 __global__ void __launch_bounds__(kScanThreads) k_level_scan(JobDev job) {
     __shared__ uint32_t wsum[kScanThreads / 32];
-    if (local_pass_timed_out(job) || !use_level_order(job)) return;
+    if (local_pass_timed_out(job)) return;
     const uint32_t l = blockIdx.x + 1, Lg = job.n_levels, n = job.n_items;
     const uint32_t per = (n + kScanThreads - 1) / kScanThreads;
     const uint32_t i0 = min(n, threadIdx.x * per), i1 = min(n, i0 + per);
@@ -414,7 +431,7 @@ __global__ void __launch_bounds__(kScanThreads) k_level_scan(JobDev job) {
 __global__ void __launch_bounds__(256) k_level_fill(JobDev job) {
     __shared__ uint32_t base[kMaxLevel + 1];
     __shared__ uint32_t cursor[8][kMaxLevel + 1];  // per warp: the block's entries written so far, per level
-    if (local_pass_timed_out(job) || !use_level_order(job)) return;
+    if (local_pass_timed_out(job)) return;
     const uint32_t Lg = job.n_levels, n = job.n_items;
     const uint32_t* tot = job.lvl_off + (uint64_t)Lg * n;
     if (threadIdx.x == 0) {
@@ -467,8 +484,6 @@ __global__ void __launch_bounds__(256) k_level_fill(JobDev job) {
     }
 }
 
-uint32_t lvl_auto_min_pieces_for(int ext_ctas) { return kWaitAllPerLane * (uint32_t)ext_ctas * kExtThreads; }
-
 cudaError_t launch_level_list(const JobDev& job, cudaStream_t st) {
     k_level_scan<<<job.n_levels, kScanThreads, 0, st>>>(job);
     cudaError_t e = cudaGetLastError();
@@ -478,14 +493,15 @@ cudaError_t launch_level_list(const JobDev& job, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// Cross-block pass in rounds.  Round 0 walks every block's pending spans (in
-// ascending order); each later round walks the spans the previous round could
-// not finish.  A span is attempted once per round and never waited on, so
-// the pass needs no ordering argument: every round finishes at least the
-// lowest pending span (its sources are final), and the number of rounds is
-// the depth of the cross-block dependency chains.  Spans finished earlier in
-// the same round are visible to later ones.  Rounds are separated by a grid
-// barrier (cooperative launch).
+// Cross-block pass.  Round 0 hands the pieces out in order and a lane waits a
+// while for sources that lower pieces are about to finish; each later round
+// walks the pieces the previous one could not finish, every piece attempted
+// once, so it needs no ordering argument: every round finishes at least the
+// lowest pending piece (its sources are final), and the number of rounds is
+// bounded by the depth of the cross-block dependency chains.  Pieces finished
+// earlier in the same round are visible to later ones.  Rounds are separated
+// by a grid barrier (cooperative launch).
+template <bool kMulti>
 __global__ void __launch_bounds__(kExtThreads) k_external(JobDev job) {
     __shared__ SpanRec recs[kExtThreads];
     __shared__ uint64_t dsts[kExtThreads];
@@ -504,16 +520,49 @@ __global__ void __launch_bounds__(kExtThreads) k_external(JobDev job) {
         job.counters[kTrace + 1] = (uint32_t)t;
         job.counters[kTrace + 2] = (uint32_t)(t >> 32);
     }
-    // round 0: pieces handed out in order; a lane waits a short while for
-    // sources that lower pieces are about to finish, then defers its piece to
-    // the rounds below.  The order is the output order (warps take blocks from
-    // a ticket, idle lanes take the block's next pieces), or, for a
-    // level-ordered job, the level list's (warps take 32 entries at a time):
-    // every level's pieces come after all pieces of the levels below, so with
-    // true level hints a lane only waits for pieces already handed out (the
-    // paper's waves, without a barrier between them).
+    // round 0: pieces handed out in order; a lane waits for the sources that
+    // lower pieces are about to finish, without limit unless wait_ns sets one:
+    // then it defers its piece to the rounds below.  The order is the output
+    // order (warps take parts of blocks from a ticket, idle lanes take the
+    // part's next pieces), or, for a level-ordered job, the level list's (warps
+    // take 32 entries at a time): every level's pieces come after all pieces of
+    // the levels below, so with true level hints a lane only waits for pieces
+    // already handed out (the paper's waves, without a barrier between them).
     {
-        const bool lv = use_level_order(job);
+        const bool lv = !kMulti && job.lvl_tab;
+        const uint64_t wait_ns = job.wait_ns == 0 || job.wait_ns == 0xffffffffu ? ~0ull : job.wait_ns;
+        uint32_t spins = 0, nap = 64;
+        uint32_t sn0 = 0;  // entries staged for list 0
+        uint64_t t0 = 0;   // start of the lane's wait (0: its piece has not been refused yet)
+        // after an attempt that left the lanes `has` waiting: pieces that have
+        // waited too long go to the rounds; a warp without progress naps.
+        // Returns false when the deadline has passed.
+        auto settle = [&](bool& has, bool progressed, uint32_t span, uint32_t item) -> bool {
+            bool giveup = false;
+            if (has) {
+                const uint64_t now = gtimer();
+                if (t0 == 0) t0 = now;
+                giveup = now - t0 > wait_ns;
+            }
+            append(giveup, ListEnt{span, item}, sbuf, sn0, job.lists[0], &job.counters[kListCnt], lane);
+            if (giveup) has = false;
+            if (__any_sync(ACX_FULL, progressed || giveup)) {
+                spins = 0;
+                nap = 64;
+                return true;
+            }
+            __nanosleep(nap);
+            if (wait_ns == ~0ull) nap = min(2 * nap, 1024u);  // long waits: fewer polls of the bitmaps
+            if ((++spins & 255) == 0 && __any_sync(ACX_FULL, gtimer() > deadline)) {
+                if (lane == 0) {
+                    const ArcJob& J = kMulti ? job.arcs[find_arc(job, item)] : job.one;
+                    set_err_arc(job, kMulti ? find_arc(job, item) : 0, kErrTimeout, kStageWait << 24,
+                                item_ref(J, item - J.item_base).blk);
+                }
+                return false;
+            }
+            return true;
+        };
         uint32_t n_lv = 0;
         if (lv) {
             n_lv = job.lvl_off[(uint64_t)job.n_levels * job.n_items + 2 * job.n_levels];  // the list's length
@@ -522,61 +571,47 @@ __global__ void __launch_bounds__(kExtThreads) k_external(JobDev job) {
                 n_lv = 0;
             }
         }
-        // wait_ns 0 (automatic): in output order, waiting pieces cost little
-        // while pieces are few per lane of the grid; with many (long, wide
-        // chains, e.g. text) waiting lanes would clog the hand-out, so a piece
-        // that waited kRound0WaitNs goes to the rounds; in level order a piece
-        // waits at most kLevelWaitNs
-        uint64_t wait_ns;
-        if (job.wait_ns == 0) {
-            wait_ns = lv ? kLevelWaitNs : few_pieces(job, (uint64_t)gridDim.x * blockDim.x) ? ~0ull : kRound0WaitNs;
-        } else {
-            wait_ns = job.wait_ns == 0xffffffffu ? ~0ull : job.wait_ns;
-        }
-        uint32_t blk = 0, dsl = 0, cnt = 0, next = 0, base = 0, item = 0;
-        int arc = 0;
-        bool exhausted = false;
-        ArcJob J = load_arc(job, 0);
-        bool has = false;
+        const uint64_t pieces = *((volatile const uint32_t*)&job.counters[kStatPending]);
+        const uint64_t per_part = (uint64_t)job.n_items * kPartPieces;
+        const uint32_t parts = (uint32_t)max((pieces + per_part - 1) / per_part, (uint64_t)1);
+        const uint64_t n_tickets = (uint64_t)job.n_items * parts;
+        uint32_t dsl = 0, cnt = 0, next = 0, base = 0, item = 0;
+        bool exhausted = false, has = false;
+        const ArcJob* J = &job.one;
+        ArcView V = view_of(job.one);  // of the lane's piece
         SpanRec rec{0, 0, 0, 0};
-        uint32_t l_blk = 0, l_dsl = 0, l_span = 0, l_item = 0;
-        int l_arc = 0;
-        uint64_t t0 = 0;
-        uint32_t spins = 0, nap = 64;
-        uint32_t sn0 = 0;  // entries staged for list 0
+        uint32_t l_dsl = 0, l_span = 0, l_item = 0;
         const uint32_t lt_mask = (1u << lane) - 1;
         for (;;) {
             uint32_t idle = __ballot_sync(ACX_FULL, !has);
             while (idle && !exhausted) {
                 if (next >= cnt) {
+                    // a level-ordered job: chunk t * kLvStripes + k of 32 entries
+                    // from stripe k's counter, so that the hand-out is not one
+                    // counter's atomics in a row (the order stays the list's, up to
+                    // how far the stripes drift apart; every CTA has warps on every
+                    // stripe).  Otherwise part t % parts of block t / parts.
+                    const uint32_t k = (threadIdx.x >> 5) & (kLvStripes - 1);
+                    uint32_t t = 0;
+                    if (lane == 0) t = atomicAdd(&job.counters[lv ? kLvTickets + k : 2], 1u);
+                    t = __shfl_sync(ACX_FULL, t, 0);
+                    next = 0;
                     if (lv) {
-                        // the next 32 entries of the level list: chunk t * kLvStripes + k
-                        // from stripe k's counter, so that the hand-out is not one
-                        // counter's atomics in a row (the order stays the list's, up to
-                        // how far the stripes drift apart)
-                        const uint32_t k = (threadIdx.x >> 5) & (kLvStripes - 1);  // (with 32 warps a CTA: every stripe in every CTA)
-                        if (lane == 0) item = atomicAdd(&job.counters[kLvTickets + k], 1u);
-                        item = (__shfl_sync(ACX_FULL, item, 0) * kLvStripes + k) * 32;
-                    } else {
-                        if (lane == 0) item = atomicAdd(&job.counters[2], 1u);
-                        item = __shfl_sync(ACX_FULL, item, 0);
-                    }
-                    if (lv) {
-                        if (item >= n_lv) { exhausted = true; break; }
-                        base = item;
-                        cnt = min(32u, n_lv - item);
-                        next = 0;
+                        base = (t * kLvStripes + k) * 32;
+                        if (base >= n_lv) { exhausted = true; break; }
+                        cnt = min(32u, n_lv - base);
                         continue;
                     }
-                    if (item >= job.n_items) { exhausted = true; break; }
-                    arc = find_arc(job, item);
-                    J = load_arc(job, arc);
-                    const ItemRef ir = item_ref(J, item - J.item_base);
-                    blk = ir.blk;
+                    if (t >= n_tickets) { exhausted = true; break; }
+                    item = t / parts;
+                    const uint32_t part = t - item * parts;
+                    if (kMulti) J = job.arcs + find_arc(job, item);
+                    const ItemRef ir = item_ref(*J, item - J->item_base);
                     dsl = ir.slot;
-                    cnt = J.npend[dsl];
-                    next = 0;
                     base = ir.span_base;
+                    const uint64_t n = J->npend[dsl];
+                    next = (uint32_t)(n * part / parts);
+                    cnt = (uint32_t)(n * (part + 1) / parts);
                     continue;
                 }
                 const uint32_t avail = cnt - next;
@@ -586,49 +621,24 @@ __global__ void __launch_bounds__(kExtThreads) k_external(JobDev job) {
                         const ListEnt e = job.lvl_list[base + next + r];
                         l_span = e.x;
                         l_item = e.y;
-                        l_blk = J.lo + e.y;  // a whole-archive job: item i is block lo + i, in slot lo + i
-                        l_dsl = l_blk;
-                        l_arc = 0;
+                        l_dsl = J->lo + e.y;  // a whole-archive job: item i is block lo + i, in slot lo + i
                     } else {
                         l_span = base + next + r;
-                        l_blk = blk;
-                        l_dsl = dsl;
                         l_item = item;
-                        l_arc = arc;
+                        l_dsl = dsl;
                     }
-                    rec = J.spans[l_span];
-                    t0 = gtimer();
+                    if (kMulti) V = view_of(*J);
+                    rec = J->spans[l_span];
+                    t0 = 0;
                     has = true;
                 }
                 next += min(avail, (uint32_t)__popc(idle));
                 idle = __ballot_sync(ACX_FULL, !has);
             }
             if (!__any_sync(ACX_FULL, has)) break;
-            // attempt the held pieces, one archive at a time
-            bool progressed = false;
-            uint32_t todo = __ballot_sync(ACX_FULL, has);
-            while (todo) {
-                const int a0 = __shfl_sync(ACX_FULL, l_arc, __ffs(todo) - 1);
-                const bool mine = has && l_arc == a0;
-                const bool done = try_pieces(mine, load_arc(job, a0), l_dsl, rec, wrec, wdst, lane);
-                if (done) { has = false; progressed = true; }
-                todo &= ~__ballot_sync(ACX_FULL, mine);
-            }
-            // give up on pieces that waited too long: the rounds finish them
-            const bool giveup = has && gtimer() - t0 > wait_ns;
-            append(giveup, ListEnt{l_span, l_item}, sbuf, sn0, job.lists[0], &job.counters[kListCnt], lane);
-            if (giveup) has = false;
-            if (__any_sync(ACX_FULL, progressed || giveup)) {
-                spins = 0;
-                nap = 64;
-            } else {
-                __nanosleep(nap);
-                if (wait_ns == ~0ull) nap = min(2 * nap, 1024u);  // long waits: fewer polls of the bitmaps
-                if ((++spins & 255) == 0 && __any_sync(ACX_FULL, gtimer() > deadline)) {
-                    if (lane == 0) set_err_arc(job, l_arc, kErrTimeout, kStageWait << 24, l_blk);
-                    break;
-                }
-            }
+            const bool done = try_pieces(has, V, l_dsl, rec, wrec, wdst, lane);
+            if (done) has = false;
+            if (__any_sync(ACX_FULL, has) && !settle(has, done, l_span, l_item)) break;
         }
         stage_flush(sbuf, sn0, job.lists[0], &job.counters[kListCnt], lane);
     }
@@ -651,10 +661,10 @@ __global__ void __launch_bounds__(kExtThreads) k_external(JobDev job) {
         if (n <= kSoloMax) {
             // a short list: one CTA finishes the remaining rounds with CTA
             // barriers instead of grid barriers
-            if (blockIdx.x == 0) solo_rounds(job, in, n, round, deadline, wrec, wdst, sbuf, lane);
+            if (blockIdx.x == 0) solo_rounds<kMulti>(job, in, n, round, deadline, wrec, wdst, sbuf, lane);
             return;
         }
-        round_pass(job, job.lists[in], out, n, gwarp, nwarps, wrec, wdst, sbuf, lane);
+        round_pass<kMulti>(job, job.lists[in], out, n, gwarp, nwarps, wrec, wdst, sbuf, lane);
     }
 }
 
@@ -728,7 +738,8 @@ cudaError_t launch_external(const JobDev& job, int grid, cudaStream_t st) {
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, k_external, *a->job);
+        return a->job->arcs ? cudaLaunchKernelEx(&cfg, k_external<true>, *a->job)
+                            : cudaLaunchKernelEx(&cfg, k_external<false>, *a->job);
     }, &a);
 }
 
@@ -742,8 +753,11 @@ int local_occupancy(size_t smem) {
 
 int external_occupancy() {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_external, kExtThreads, 0) != cudaSuccess) return 0;
-    return n;
+    int m = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_external<false>, kExtThreads, 0) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, k_external<true>, kExtThreads, 0) != cudaSuccess)
+        return 0;
+    return std::min(n, m);
 }
 
 }  // namespace acx

@@ -165,12 +165,6 @@ __device__ __forceinline__ ItemRef item_ref(const ArcJob& J, uint32_t idx) {
     }
     return r;
 }
-// Output slot of block a, and the output offset of absolute position pos.
-__device__ __forceinline__ uint64_t slot_of(const ArcJob& J, uint64_t a) { return J.slot ? J.slot[a] : a; }
-__device__ __forceinline__ uint64_t out_off(const ArcJob& J, uint64_t pos) {
-    return J.slot ? (uint64_t)J.slot[pos >> 14] * kBlock + (pos & (kBlock - 1)) : pos;
-}
-
 // Is block id a in the ascending list dl[0, n)?
 __device__ __forceinline__ bool listed(const uint32_t* dl, uint32_t n, uint32_t a) {
     uint32_t lo = 0, hi = n;

@@ -119,7 +119,6 @@ struct LaunchPlan {
 // which the default variant may do with the fused entropy + local kernel.
 int launch_plan(aceapex_ctx* c, const aceapex_dec_params& p, uint32_t max_tok, uint32_t max_lenb, LaunchPlan* lp,
                 uint32_t job_flags = 0, bool whole_single = false);
-inline uint32_t lvl_auto_min_pieces(const aceapex_ctx* c) { return lvl_auto_min_pieces_for(c->occ_ext * c->n_sms); }
 // Synchronise st and return (and clear) the context's device error status.
 int ctx_read_status(aceapex_ctx* c, cudaStream_t st);
 

@@ -169,7 +169,6 @@ struct JobDev {
     uint32_t* lvl_off;
     ListEnt* lvl_list;
     uint32_t lvl_cap;         // entries lvl_list holds
-    uint32_t lvl_min_pieces;  // automatic policy (wait_ns 0): level order only above this many pending pieces
 };
 constexpr uint32_t kMaxLevel = 255;
 

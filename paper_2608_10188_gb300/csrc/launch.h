@@ -24,9 +24,6 @@ cudaError_t coop_ordered(cudaStream_t st, cudaError_t (*launch)(void*), void* ar
 // The level list of a level-ordered job (kJobLevels): a per-level scan over
 // the items, then one warp per item writes its pieces' entries.
 cudaError_t launch_level_list(const JobDev& job, cudaStream_t st);
-// Pending pieces above which the automatic policy takes a level-ordered job's
-// pieces in level order: 16 per thread of the cross-block pass's grid.
-uint32_t lvl_auto_min_pieces_for(int ext_ctas);
 cudaError_t launch_plain(const JobDev& job, int grid, cudaStream_t st);
 // Fused entropy stage + local pass of a whole single-archive job (job.ready
 // set, its flags cleared): G local groups per CTA, one CTA per SM
