@@ -275,6 +275,7 @@ static int enqueue_decode(aceapex_ctx* c, aceapex_archive* A, const void* d_arc,
     job.timeout_ns = (uint64_t)c->params.timeout_us * 1000ull;
     job.max_tok = P.max_tok;
     job.max_lenb = P.max_lenb;
+    job.max_lit = P.max_lit;
     job.lists[0] = (JobDev::ListEnt*)c->lists.p;
     job.lists[1] = (JobDev::ListEnt*)c->lists.p + std::max<uint64_t>(P.span_slots, 1);
     if (hi <= lo) return ACEAPEX_OK;
@@ -295,7 +296,7 @@ static int enqueue_decode(aceapex_ctx* c, aceapex_archive* A, const void* d_arc,
         job.flags |= kJobLevels;
     }
     LaunchPlan lp;
-    int rc = launch_plan(c, c->params, P.max_tok, P.max_lenb, &lp, job.flags, true);
+    int rc = launch_plan(c, c->params, P.max_tok, P.max_lenb, P.max_lit, &lp, job.flags, true);
     if (rc) return rc;
     if (lp.fused_groups) {
         if ((e = c->ready.ensure(nb * 4)) != cudaSuccess) return cuda_fail(c, e, "ready-flag allocation");
@@ -305,7 +306,7 @@ static int enqueue_decode(aceapex_ctx* c, aceapex_archive* A, const void* d_arc,
 }
 
 int acx::launch_plan(aceapex_ctx* c, const aceapex_dec_params& p, uint32_t max_tok, uint32_t max_lenb,
-                     LaunchPlan* lp, uint32_t job_flags, bool whole_single) {
+                     uint32_t max_lit, LaunchPlan* lp, uint32_t job_flags, bool whole_single) {
     // parse-only and wanted-byte jobs run the scan decoder (the serial one has neither mode)
     lp->variant = (job_flags & (kJobIndex | kJobNeed)) ? (uint32_t)ACEAPEX_VARIANT_FAST : p.variant;
     if (lp->variant > ACEAPEX_VARIANT_FUSED) return fail(c, ACEAPEX_E_ARG, "unknown decoder variant");
@@ -317,7 +318,7 @@ int acx::launch_plan(aceapex_ctx* c, const aceapex_dec_params& p, uint32_t max_t
     lp->grid_local = 0;
     if (lp->variant != ACEAPEX_VARIANT_PLAIN) {
         const size_t lsm =
-            local_smem_bytes(max_tok, max_lenb, (job_flags & kJobNeed) != 0, (job_flags & kJobLevels) != 0);
+            local_smem_bytes(max_tok, max_lenb, max_lit, (job_flags & kJobNeed) != 0, (job_flags & kJobLevels) != 0);
         if (lsm > 227 * 1024) return fail(c, ACEAPEX_E_CORRUPT, "block too large for the local pass");
         if (c->occ_local_smem != lsm) {  // (an occupancy query per launch costs the serving ticks host time)
             c->occ_local = local_occupancy(lsm);
@@ -331,8 +332,8 @@ int acx::launch_plan(aceapex_ctx* c, const aceapex_dec_params& p, uint32_t max_t
     // job is one whole archive and a CTA holds the tables and a workspace
     if (whole_single && lp->variant == ACEAPEX_VARIANT_FUSED && !(job_flags & (kJobIndex | kJobNeed))) {
         const bool lvl = (job_flags & kJobLevels) != 0;
-        const int G = fused_groups(max_tok, max_lenb, lvl);
-        if (G > 0 && fused_occupancy(G, max_tok, max_lenb, lvl) >= 1) {
+        const int G = fused_groups(max_tok, max_lenb, max_lit, lvl);
+        if (G > 0 && fused_occupancy(G, max_tok, max_lenb, max_lit, lvl) >= 1) {
             lp->fused_groups = G;
             lp->grid_fused = c->n_sms;
         }

@@ -38,9 +38,10 @@
 
 namespace acx {
 
-__global__ void __launch_bounds__(kLocThreads, 6) k_local(JobDev job) {
+template <int NT>
+__global__ void __launch_bounds__(NT, NT == kLocThreads ? 6 : NT == kLocWide ? 3 : 1) k_local(JobDev job) {
     extern __shared__ __align__(128) uint8_t sm[];
-    local_worker(job, sm, 0, threadIdx.x);
+    local_worker<NT>(job, sm, 0, threadIdx.x);
 }
 
 // ---- cross-block pass --------------------------------------------------------------------
@@ -668,20 +669,51 @@ __global__ void __launch_bounds__(kExtThreads) k_external(JobDev job) {
     }
 }
 
-size_t local_smem_bytes(uint32_t T, uint32_t LB, bool need, bool lvl) { return loc_layout(T, LB, need, lvl).total; }
+size_t local_smem_bytes(uint32_t T, uint32_t LB, uint32_t LIT, bool need, bool lvl) {
+    return loc_layout(T, LB, LIT, need, lvl).total;
+}
+
+// Threads of a local CTA for a job of n_items blocks of up to T tokens whose
+// workspace has `smem` bytes.  A CTA's shared memory sets how many fit an SM:
+// with four or fewer (blocks of some 900 tokens and more), 128 threads leave
+// most of the SM's issue slots empty (200 MiB text: 487 us; 256 threads 461; a
+// batch of 96 files 936 -> 825), with five or six they fill it (254 MB genome:
+// 322 us; 256 threads 420).  A job of few blocks has every block on an SM at
+// once, so only a block's latency counts: 256 threads, or 512 for blocks of
+// many tokens (4 MiB DNA-like 34 -> 27 us; 4 MiB text 97 -> 73 -> 60 with 128,
+// 256, 512 threads; one 10 KB text block 62 -> 43 -> 35).
+static int local_threads(size_t smem, uint32_t n_items, uint32_t T) {
+    if (n_items <= 2u * (uint32_t)noted_sm_count()) return T > 256 ? kLocWidest : kLocWide;
+    return 227 * 1024 / (smem + 1024) <= 4 ? kLocWide : kLocThreads;
+}
+
+template <int NT>
+static cudaError_t local_attrs(size_t smem) {
+    cudaError_t e = cudaFuncSetAttribute(k_local<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)  // the whole unified L1 as shared memory: CTAs per SM are set by their workspaces
+        e = cudaFuncSetAttribute(k_local<NT>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 cudaSharedmemCarveoutMaxShared);
+    return e;
+}
+
+template <int NT>
+static cudaError_t launch_local_nt(const JobDev& job, int grid, size_t smem, cudaStream_t st) {
+    const cudaError_t e = local_attrs<NT>(smem);
+    if (e != cudaSuccess) return e;
+    k_local<NT><<<grid, NT, smem, st>>>(job);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_local(const JobDev& job, int grid, cudaStream_t st) {
-    const size_t sm = local_smem_bytes(job.max_tok, job.max_lenb, (job.flags & kJobNeed) != 0,
+    const size_t sm = local_smem_bytes(job.max_tok, job.max_lenb, job.max_lit, (job.flags & kJobNeed) != 0,
                                        (job.flags & kJobLevels) != 0);
-    cudaError_t e = cudaFuncSetAttribute(k_local, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e == cudaSuccess)  // the whole unified L1 as shared memory: CTAs per SM are set by their workspaces
-        e = cudaFuncSetAttribute(k_local, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
     // a small job (a seek, a serving tick) needs no more CTAs than ticket runs
     const uint64_t runs = (job.n_items + (uint64_t)(job.chunk ? job.chunk : 1) - 1) / (job.chunk ? job.chunk : 1);
     grid = job_grid(grid, runs);
-    k_local<<<grid, kLocThreads, sm, st>>>(job);
-    return cudaGetLastError();
+    const int nt = local_threads(sm, job.n_items, job.max_tok);
+    return nt == kLocWidest ? launch_local_nt<kLocWidest>(job, grid, sm, st)
+           : nt == kLocWide ? launch_local_nt<kLocWide>(job, grid, sm, st)
+                            : launch_local_nt<kLocThreads>(job, grid, sm, st);
 }
 
 // Cooperative launches (the cross-block pass, the fused decode) run one at a
@@ -743,12 +775,18 @@ cudaError_t launch_external(const JobDev& job, int grid, cudaStream_t st) {
     }, &a);
 }
 
-int local_occupancy(size_t smem) {
-    cudaFuncSetAttribute(k_local, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_local, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+template <int NT>
+static int local_occupancy_nt(size_t smem) {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_local, kLocThreads, smem) != cudaSuccess) return 0;
+    if (local_attrs<NT>(smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_local<NT>, NT, smem) != cudaSuccess)
+        return 0;
     return n;
+}
+
+int local_occupancy(size_t smem) {  // (of a job of many blocks: a small one fits an SM or two per block)
+    return local_threads(smem, 0xffffffffu, 0) == kLocWide ? local_occupancy_nt<kLocWide>(smem)
+                                                           : local_occupancy_nt<kLocThreads>(smem);
 }
 
 int external_occupancy() {

@@ -71,7 +71,7 @@ int aceapex_batch_create(aceapex_ctx* c, const aceapex_batch_item* items, int n,
     std::vector<ArcJob> tab(std::max(n, 1));
     std::vector<uint64_t> o_str(n), o_np(n), o_pm(n), o_sp(n);
     uint64_t s_str = 0, s_np = 0, s_pm = 0, s_sp = 0, slots = 0, items_total = 0;
-    uint32_t max_tok = 0, max_lenb = 0;
+    uint32_t max_tok = 0, max_lenb = 0, max_lit = 0;
     for (int a = 0; a < n; a++) {
         const aceapex_archive* A = items[a].arc;
         if (!A || (!items[a].d_out && A->plan.total)) {
@@ -99,6 +99,7 @@ int aceapex_batch_create(aceapex_ctx* c, const aceapex_batch_item* items, int n,
         items_total += P.n_blocks;
         max_tok = std::max(max_tok, P.max_tok);
         max_lenb = std::max(max_lenb, P.max_lenb);
+        max_lit = std::max(max_lit, P.max_lit);
         B->bytes += P.total;
     }
     if (items_total >= 0xffffffffull) {
@@ -106,7 +107,7 @@ int aceapex_batch_create(aceapex_ctx* c, const aceapex_batch_item* items, int n,
         return fail(c, ACEAPEX_E_ARG, "batch_create: too many blocks in one batch");
     }
     B->blocks = items_total;
-    int rc = launch_plan(c, c->params, max_tok, max_lenb, &B->lp);
+    int rc = launch_plan(c, c->params, max_tok, max_lenb, max_lit, &B->lp);
     if (rc) {
         batch_free(B);
         return rc;
@@ -163,6 +164,7 @@ int aceapex_batch_create(aceapex_ctx* c, const aceapex_batch_item* items, int n,
     job.timeout_ns = (uint64_t)c->params.timeout_us * 1000ull;
     job.max_tok = max_tok;
     job.max_lenb = max_lenb;
+    job.max_lit = max_lit;
     job.lists[0] = (JobDev::ListEnt*)(base + r_ls);
     job.lists[1] = job.lists[0] + slots;
     B->h_errs.assign(4 + n, 0);
@@ -307,7 +309,7 @@ extern "C" int aceapex_autotune(aceapex_ctx* c, const aceapex_batch_item* items,
         if (flush) cudaFree(flush);
         return cuda_fail(c, e, "autotune");
     }
-    const size_t lsm = local_smem_bytes(B->job.max_tok, B->job.max_lenb);
+    const size_t lsm = local_smem_bytes(B->job.max_tok, B->job.max_lenb, B->job.max_lit);
     const int occ_local = base.variant == ACEAPEX_VARIANT_PLAIN ? 1 : std::max(1, local_occupancy(lsm));
     std::vector<uint32_t> locals, ranss;
     for (int v : {1, 2, 3, 4, 6, 8, 12, 16})
@@ -326,7 +328,7 @@ extern "C" int aceapex_autotune(aceapex_ctx* c, const aceapex_batch_item* items,
                 p.rans_ctas_per_sm = rcn;
                 p.queue_chunk = ch;
                 LaunchPlan lp;
-                if ((rc = launch_plan(c, p, B->job.max_tok, B->job.max_lenb, &lp))) break;
+                if ((rc = launch_plan(c, p, B->job.max_tok, B->job.max_lenb, B->job.max_lit, &lp))) break;
                 B->lp = lp;
                 t.clear();
                 for (int r = 0; r <= reps && rc == ACEAPEX_OK; r++) {

@@ -145,7 +145,7 @@ int acx::build_match_index(aceapex_ctx* c, aceapex_archive* A) {
         const uint32_t c1 = std::min(P.n_blocks, c0 + kChunk), k = c1 - c0;
         it.assign(k, ItemDev{});
         uint64_t toks = 0, sb = 0;
-        uint32_t max_tok = 1, max_lenb = 1;
+        uint32_t max_tok = 1, max_lenb = 1, max_lit = 0;
         for (uint32_t i = 0; i < k; i++) {
             const BlockDev& bd = P.blk[c0 + i];
             it[i].block = c0 + i;
@@ -156,6 +156,7 @@ int acx::build_match_index(aceapex_ctx* c, aceapex_archive* A) {
             sb += (bd.s_off[3] + bd.s_raw[3] + 15) & ~15ull;
             max_tok = std::max(max_tok, bd.n_tok);
             max_lenb = std::max(max_lenb, bd.s_raw[kLen]);
+            max_lit = std::max(max_lit, bd.s_raw[kLit]);
         }
         sb += 64;
         if ((e = items.ensure(k * sizeof(ItemDev))) != cudaSuccess ||
@@ -188,9 +189,10 @@ int acx::build_match_index(aceapex_ctx* c, aceapex_archive* A) {
         job.timeout_ns = (uint64_t)c->params.timeout_us * 1000ull;
         job.max_tok = max_tok;
         job.max_lenb = max_lenb;
+        job.max_lit = max_lit;
         job.flags = kJobIndex;
         LaunchPlan lp;
-        if ((rc = launch_plan(c, c->params, max_tok, max_lenb, &lp, kJobIndex))) break;
+        if ((rc = launch_plan(c, c->params, max_tok, max_lenb, max_lit, &lp, kJobIndex))) break;
         if ((rc = enqueue_job(c, job, lp, 4, nullptr, 0, st, nullptr))) break;
         // a corrupt block is recorded in its status word and the index goes on
         if ((rc = ctx_read_status(c, st)) && rc != ACEAPEX_E_CORRUPT) break;

@@ -29,15 +29,16 @@ namespace acx {
 
 constexpr int kFusedRansWarps = 12;
 constexpr int kFusedMaxGroups = 3;
-constexpr int kFusedMaxThreads = 32 * (kFusedRansWarps + kLocWarps * kFusedMaxGroups);
+constexpr int kGroupWarps = kLocThreads / 32;
+constexpr int kFusedMaxThreads = 32 * (kFusedRansWarps + kGroupWarps * kFusedMaxGroups);
 
 struct FusedLayout {
     uint32_t tab, ring, bar, stage, loc, loc_stride, total;
 };
 
 // Shared memory of a fused CTA with G local groups whose workspaces hold
-// blocks of up to T tokens and LB length bytes.
-__host__ __device__ inline FusedLayout fused_layout(uint32_t T, uint32_t LB, int G, bool lvl) {
+// blocks of up to T tokens, LB length bytes and LIT literals.
+__host__ __device__ inline FusedLayout fused_layout(uint32_t T, uint32_t LB, uint32_t LIT, int G, bool lvl) {
     FusedLayout F;
     F.tab = 0;                                           // 4 x 4096 decode entries
     F.ring = 4 * kM * 4;                                 // (R + 1) x 2 KiB: R rings, 2 KiB-aligned inside
@@ -45,7 +46,7 @@ __host__ __device__ inline FusedLayout fused_layout(uint32_t T, uint32_t LB, int
     F.stage = F.bar + kFusedRansWarps * (kSlots + 1) * 8;  // R x kStageBytes symbol stages (16-aligned)
     const uint32_t end = F.stage + kFusedRansWarps * kStageBytes;
     F.loc = (end + 127) & ~127u;
-    F.loc_stride = loc_layout(T, LB, false, lvl).total;  // 128-byte multiple
+    F.loc_stride = loc_layout(T, LB, LIT, false, lvl).total;  // 128-byte multiple
     F.total = F.loc + (uint32_t)G * F.loc_stride;
     return F;
 }
@@ -56,7 +57,7 @@ __device__ __forceinline__ void st_release_u32(uint32_t* p, uint32_t v) {
 
 __global__ void __launch_bounds__(kFusedMaxThreads, 1) k_fused(JobDev job, int G) {
     extern __shared__ __align__(128) uint8_t sm[];
-    const FusedLayout F = fused_layout(job.max_tok, job.max_lenb, G, (job.flags & kJobLevels) != 0);
+    const FusedLayout F = fused_layout(job.max_tok, job.max_lenb, job.max_lit, G, (job.flags & kJobLevels) != 0);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const ArcJob& J = job.one;
     {
@@ -94,19 +95,19 @@ __global__ void __launch_bounds__(kFusedMaxThreads, 1) k_fused(JobDev job, int G
         }
         return;
     }
-    const int g = (warp - kFusedRansWarps) / kLocWarps;
+    const int g = (warp - kFusedRansWarps) / kGroupWarps;
     if (g >= G) return;
-    local_worker(job, sm + F.loc + g * F.loc_stride, 1 + g, threadIdx.x - 32 * (kFusedRansWarps + kLocWarps * g));
+    local_worker<kLocThreads>(job, sm + F.loc + g * F.loc_stride, 1 + g, threadIdx.x - 32 * (kFusedRansWarps + kGroupWarps * g));
 }
 
-int fused_groups(uint32_t max_tok, uint32_t max_lenb, bool lvl) {
+int fused_groups(uint32_t max_tok, uint32_t max_lenb, uint32_t max_lit, bool lvl) {
     for (int G = kFusedMaxGroups; G >= 1; G--)
-        if (fused_layout(max_tok, max_lenb, G, lvl).total <= 227u * 1024) return G;
+        if (fused_layout(max_tok, max_lenb, max_lit, G, lvl).total <= 227u * 1024) return G;
     return 0;
 }
 
 cudaError_t launch_fused(const JobDev& job, int G, int grid, cudaStream_t st) {
-    const FusedLayout F = fused_layout(job.max_tok, job.max_lenb, G, (job.flags & kJobLevels) != 0);
+    const FusedLayout F = fused_layout(job.max_tok, job.max_lenb, job.max_lit, G, (job.flags & kJobLevels) != 0);
     cudaError_t e = cudaFuncSetAttribute(k_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F.total);
     if (e != cudaSuccess) return e;
     struct Arg {
@@ -119,7 +120,7 @@ cudaError_t launch_fused(const JobDev& job, int G, int grid, cudaStream_t st) {
         const Arg* a = static_cast<const Arg*>(p);
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(a->grid);
-        cfg.blockDim = dim3(32 * (kFusedRansWarps + kLocWarps * a->G));
+        cfg.blockDim = dim3(32 * (kFusedRansWarps + kGroupWarps * a->G));
         cfg.dynamicSmemBytes = a->smem;
         cfg.stream = a->st;
         cudaLaunchAttribute attr[1];
@@ -131,12 +132,12 @@ cudaError_t launch_fused(const JobDev& job, int G, int grid, cudaStream_t st) {
     }, &a);
 }
 
-int fused_occupancy(int G, uint32_t max_tok, uint32_t max_lenb, bool lvl) {
-    const FusedLayout F = fused_layout(max_tok, max_lenb, G, lvl);
+int fused_occupancy(int G, uint32_t max_tok, uint32_t max_lenb, uint32_t max_lit, bool lvl) {
+    const FusedLayout F = fused_layout(max_tok, max_lenb, max_lit, G, lvl);
     if (cudaFuncSetAttribute(k_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F.total) != cudaSuccess)
         return 0;
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused, 32 * (kFusedRansWarps + kLocWarps * G), F.total) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused, 32 * (kFusedRansWarps + kGroupWarps * G), F.total) !=
         cudaSuccess)
         return 0;
     return n;

@@ -113,12 +113,12 @@ struct LaunchPlan {
     int grid_rans = 0, grid_local = 0, grid_plain = 0, grid_ext = 0;
     int fused_groups = 0, grid_fused = 0;  // fused entropy + local pass (whole single-archive jobs), 0: staged
 };
-// Grids for a job whose largest block has max_tok tokens and max_lenb length
-// bytes, under decoder parameters p (fails when a block cannot fit the local
+// Grids for a job whose largest block has max_tok tokens, max_lenb length
+// bytes and max_lit literals, under decoder parameters p (fails when a block cannot fit the local
 // pass's shared memory).  whole_single: the job decodes one whole archive,
 // which the default variant may do with the fused entropy + local kernel.
-int launch_plan(aceapex_ctx* c, const aceapex_dec_params& p, uint32_t max_tok, uint32_t max_lenb, LaunchPlan* lp,
-                uint32_t job_flags = 0, bool whole_single = false);
+int launch_plan(aceapex_ctx* c, const aceapex_dec_params& p, uint32_t max_tok, uint32_t max_lenb, uint32_t max_lit,
+                LaunchPlan* lp, uint32_t job_flags = 0, bool whole_single = false);
 // Synchronise st and return (and clear) the context's device error status.
 int ctx_read_status(aceapex_ctx* c, cudaStream_t st);
 
@@ -133,7 +133,7 @@ void block_closure(aceapex_archive* A, uint32_t b0, uint32_t b1, std::vector<uin
 struct SubsetPlan {
     std::vector<ItemDev> items;
     uint64_t scratch_bytes = 0, span_slots = 0;
-    uint32_t max_tok = 1, max_lenb = 1;
+    uint32_t max_tok = 1, max_lenb = 1, max_lit = 0;
 };
 void subset_plan(const Plan& P, const uint32_t* blocks, const uint32_t* slots, size_t n, SubsetPlan* S);
 

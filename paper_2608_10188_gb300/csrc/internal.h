@@ -145,6 +145,7 @@ struct JobDev {
     uint64_t timeout_ns;
     uint32_t max_tok;         // shared-memory sizing of the assembly kernel
     uint32_t max_lenb;
+    uint32_t max_lit;
     uint32_t flags;           // kJob* bits
     uint32_t chunk;           // work items per ticket of the entropy stage and the local pass (0 = 1)
     uint32_t wait_ns;         // cross-block round 0: how long a piece may wait for its sources before it

@@ -28,11 +28,12 @@ cudaError_t launch_plain(const JobDev& job, int grid, cudaStream_t st);
 // Fused entropy stage + local pass of a whole single-archive job (job.ready
 // set, its flags cleared): G local groups per CTA, one CTA per SM
 // (cooperative).  fused_groups: the most groups whose workspaces fit a CTA
-// for blocks of max_tok tokens and max_lenb length bytes (0: none fits).
+// for blocks of max_tok tokens, max_lenb length bytes and max_lit
+// literals (0: none fits).
 cudaError_t launch_fused(const JobDev& job, int G, int grid, cudaStream_t st);
-int fused_groups(uint32_t max_tok, uint32_t max_lenb, bool lvl);
-int fused_occupancy(int G, uint32_t max_tok, uint32_t max_lenb, bool lvl);
-size_t local_smem_bytes(uint32_t T, uint32_t LB, bool need = false, bool lvl = false);
+int fused_groups(uint32_t max_tok, uint32_t max_lenb, uint32_t max_lit, bool lvl);
+int fused_occupancy(int G, uint32_t max_tok, uint32_t max_lenb, uint32_t max_lit, bool lvl);
+size_t local_smem_bytes(uint32_t T, uint32_t LB, uint32_t LIT, bool need = false, bool lvl = false);
 int rans_occupancy();
 // Grid of a persistent kernel for a job that can use `need` CTAs at most:
 // no more than `full`, and no fewer than one per SM, so that a mid-size job
@@ -41,6 +42,7 @@ int rans_occupancy();
 // which may be inside a graph capture).
 int job_grid(int full, uint64_t need);
 void note_sm_count(int n_sms);
+int noted_sm_count();
 int local_occupancy(size_t smem);
 int external_occupancy();
 int plain_occupancy();

@@ -6,18 +6,20 @@
 
 namespace acx {
 
-constexpr int kLocThreads = 128;
-constexpr int kLocWarps = kLocThreads / 32;
+// Threads of a local group: 128 when a block's workspace leaves room for five
+// CTAs or more per SM, else 256 or 512 (see local_threads).
+constexpr int kLocThreads = 128, kLocWide = 256, kLocWidest = 512;
+constexpr int kLocMaxWarps = kLocWidest / 32;
 
 struct LocLayout {
     uint32_t out, pend, tsrc, tpos, tll, tml, tlit, tcmd, tstat, lenb, soff, slit, scan, bar, misc, need, tlvl, tlvk,
         lhist, total;
 };
 
-// Shared-memory workspace of one local group for blocks of up to T tokens
-// and LB length bytes; need: jobs with wanted-byte intervals; lvl: jobs that
+// Shared-memory workspace of one local group for blocks of up to T tokens,
+// LB length bytes and LIT literals; need: jobs with wanted-byte intervals; lvl: jobs that
 // sort pieces by level (the token levels and a level histogram).
-__host__ __device__ inline LocLayout loc_layout(uint32_t T, uint32_t LB, bool need, bool lvl = false) {
+__host__ __device__ inline LocLayout loc_layout(uint32_t T, uint32_t LB, uint32_t LIT, bool need, bool lvl = false) {
     LocLayout L;
     uint32_t o = 0;
     auto take = [&](uint32_t bytes, uint32_t align) {
@@ -38,8 +40,8 @@ __host__ __device__ inline LocLayout loc_layout(uint32_t T, uint32_t LB, bool ne
     L.tstat = take(T16, 16);
     L.lenb = take(((LB + 15) & ~15u) + 16, 16);
     L.soff = take(((5 * T + 15) & ~15u) + 16, 16);
-    L.slit = take(kBlock + 16, 16);
-    L.scan = take(kLocWarps * 4 * 4 + 64, 16);
+    L.slit = take(((LIT + 15) & ~15u) + 16, 16);
+    L.scan = take(kLocMaxWarps * 3 * 4, 16);
     L.bar = take(8, 8);
     L.misc = take(64, 16);
     L.need = need ? take(kBlock / 8, 16) : 0;  // wanted-byte bitmap (jobs with kJobNeed)
@@ -61,24 +63,27 @@ __device__ __forceinline__ bool wanted(const uint32_t* need, uint32_t o, uint32_
     return false;
 }
 
-// Barriers of one 128-thread group: named barrier `bid` (0 in k_local, where
+// Barriers of one group of NT threads: named barrier `bid` (0 in k_local, where
 // the group is the whole CTA; 1.. for the groups of a fused CTA).
+template <int NT>
 __device__ __forceinline__ void grp_sync(uint32_t bid) {
-    asm volatile("bar.sync %0, %1;" ::"r"(bid), "n"(kLocThreads) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"r"(bid), "n"(NT) : "memory");
 }
+template <int NT>
 __device__ __forceinline__ int grp_or(uint32_t bid, int v) {
     uint32_t r;
     asm volatile(
         "{\n .reg .pred p, q;\n setp.ne.u32 q, %1, 0;\n barrier.cta.red.or.pred p, %2, %3, q;\n"
         " selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(r)
-        : "r"((uint32_t)v), "r"(bid), "n"(kLocThreads)
+        : "r"((uint32_t)v), "r"(bid), "n"(NT)
         : "memory");
     return (int)r;
 }
 
 // Group-wide exclusive scan of three u32 values per thread (tid: the thread
 // in its group).
+template <int NT>
 __device__ __forceinline__ void block_scan3(uint32_t v[3], uint32_t tot[3], uint32_t* buf, uint32_t bid, int tid) {
     const int lane = tid & 31, warp = tid >> 5;
     uint32_t inc[3] = {v[0], v[1], v[2]};
@@ -92,10 +97,10 @@ __device__ __forceinline__ void block_scan3(uint32_t v[3], uint32_t tot[3], uint
     }
     if (lane == 31)
         for (int k = 0; k < 3; k++) buf[warp * 3 + k] = inc[k];
-    grp_sync(bid);
+    grp_sync<NT>(bid);
     uint32_t wpre[3] = {0, 0, 0}, t[3] = {0, 0, 0};
 #pragma unroll
-    for (int w = 0; w < kLocWarps; w++) {
+    for (int w = 0; w < (NT / 32); w++) {
 #pragma unroll
         for (int k = 0; k < 3; k++) {
             const uint32_t s = buf[w * 3 + k];
@@ -108,7 +113,7 @@ __device__ __forceinline__ void block_scan3(uint32_t v[3], uint32_t tot[3], uint
         v[k] = wpre[k] + inc[k] - v[k];
         tot[k] = t[k];
     }
-    grp_sync(bid);
+    grp_sync<NT>(bid);
 }
 
 // The four-entry distance history ("The Last Sequential Element") as a map
@@ -200,7 +205,7 @@ __device__ __forceinline__ void stage_streams(const JobDev& job, uint32_t item, 
     const ItemRef ir = item_ref(J, item - J.item_base);
     const BlockDev& bd = J.blk[ir.blk];
     const uint32_t n = bd.n_tok, LB = bd.s_raw[kLen], n_new = bd.n_new, n_lit = bd.s_raw[kLit];
-    if (n > job.max_tok || LB > job.max_lenb || n_new > job.max_tok || n_lit > kBlock) return;
+    if (n > job.max_tok || LB > job.max_lenb || n_new > job.max_tok || n_lit > job.max_lit) return;
     const uint8_t* scr = J.scratch + ir.scratch;
     const uint32_t sz[4] = {(n + 15) & ~15u, (LB + 15) & ~15u, (5 * n_new + 15) & ~15u, (n_lit + 15) & ~15u};
     uint8_t* dsts[4] = {tcmd, lenb, soff, slit};
@@ -234,12 +239,13 @@ __device__ __forceinline__ bool wait_ready(const uint32_t* ready, uint32_t item,
     return true;
 }
 
-// The local pass of one 128-thread group (k_local: a whole CTA; k_fused: a
+// The local pass of one group of NT threads (k_local: a whole CTA; k_fused: a
 // group of a fused CTA) over the job's tickets, with its workspace at sm and
 // named barrier bid; tid is the thread's index in its group.
+template <int NT>
 __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uint32_t bid, int tid) {
     const bool lvl = (job.flags & kJobLevels) != 0;
-    const LocLayout L = loc_layout(job.max_tok, job.max_lenb, (job.flags & kJobNeed) != 0, lvl);
+    const LocLayout L = loc_layout(job.max_tok, job.max_lenb, job.max_lit, (job.flags & kJobNeed) != 0, lvl);
     uint8_t* tlvl = sm + L.tlvl;                                      // valid in kJobLevels jobs
     uint8_t* tlvk = sm + L.tlvk;
     uint32_t* lhist = reinterpret_cast<uint32_t*>(sm + L.lhist);
@@ -264,7 +270,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
     const uint64_t copy_deadline = gtimer() + kCopyWaitNs;    // waits on this group's own bulk copies
     if (tid == 0) mbar_init(bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    grp_sync(bid);
+    grp_sync<NT>(bid);
     uint32_t phase = 0;
     const uint32_t chunk = job.chunk ? job.chunk : 1u;
     uint32_t cnext = 0, cleft = 0;  // the group's current run of `chunk` tickets
@@ -280,7 +286,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
         } else {
             if (cleft == 0) {
                 if (tid == 0) misc[0] = atomicAdd(&job.counters[1], chunk);
-                grp_sync(bid);
+                grp_sync<NT>(bid);
                 cnext = misc[0];
                 cleft = chunk;
             }
@@ -297,7 +303,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
         auto settle_claim = [&]() {
             if (!claimed) return;
             if (tid == 0) misc[0] = pre_claim;
-            grp_sync(bid);
+            grp_sync<NT>(bid);
             cnext = misc[0];
             cleft = chunk;
             claimed = false;
@@ -311,7 +317,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
         const uint64_t B = (uint64_t)b * kBlock;
         const uint32_t R = bd.raw_len, n = bd.n_tok, LB = bd.s_raw[kLen], n_lit = bd.s_raw[kLit];
         const uint32_t n_new = bd.n_new;
-        bool bad = n > job.max_tok || LB > job.max_lenb || n_new > job.max_tok || n_lit > kBlock;
+        bool bad = n > job.max_tok || LB > job.max_lenb || n_new > job.max_tok || n_lit > job.max_lit;
         int stage = bad ? kStageLimits : 0;
         auto mark = [&](bool cond, int st) {
             if (cond && !bad) { bad = true; stage = st; }
@@ -321,18 +327,18 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
         //      they were prefetched during the previous block) ----
         if (!bad && tid == 0 && !prefetched && (!job.ready || wait_ready(job.ready, item, deadline)))
             stage_streams(job, item, tcmd, lenb, soff, slit, tlvl, bar);
-        for (uint32_t i = tid; i < kBlock / 32; i += kLocThreads) pend[i] = 0;
+        for (uint32_t i = tid; i < kBlock / 32; i += NT) pend[i] = 0;
         if (tid == 0) misc[1] = 0;
         // wanted bytes of this item (all when it names none)
         const bool partial = (job.flags & kJobNeed) && ir.need_n != 0;
         if (partial) {
-            for (uint32_t i = tid; i < kBlock / 32; i += kLocThreads) need[i] = 0;
-            grp_sync(bid);
+            for (uint32_t i = tid; i < kBlock / 32; i += NT) need[i] = 0;
+            grp_sync<NT>(bid);
             for (uint32_t q = 0; q < ir.need_n; q++) {
                 const uint32_t iv = J.need[ir.need_off + q];
                 const uint32_t s0 = iv & 0xffff, e0 = min(iv >> 16, kBlock);
                 if (s0 < e0)
-                    for (uint32_t w = (s0 >> 5) + tid; w <= ((e0 - 1) >> 5); w += kLocThreads)
+                    for (uint32_t w = (s0 >> 5) + tid; w <= ((e0 - 1) >> 5); w += NT)
                         atomicOr(&need[w], range_mask(w, s0, e0));
             }
         }
@@ -343,7 +349,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 if ((++spins & 1023) == 0 && gtimer() > copy_deadline) { timed_out = true; break; }
             phase++;
         }
-        if (grp_or(bid, timed_out)) {
+        if (grp_or<NT>(bid, timed_out)) {
             // a copy that never lands: give up on the decode (the barrier phase is lost)
             if (tid == 0) set_err_arc(job, a, kErrTimeout, kStageWait << 24, b);
             return;
@@ -351,7 +357,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
 
         // ---- varints: each byte < 0x80 ends a value ----
         uint32_t v3[3], tot3[3];
-        const uint32_t per = (LB + kLocThreads - 1) / kLocThreads;
+        const uint32_t per = (LB + NT - 1) / NT;
         const uint32_t j0 = min(LB, tid * per), j1 = min(LB, j0 + per);
         {
             uint32_t c = 0;
@@ -365,7 +371,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 }
             if (vbad) misc[1] = 1;
             v3[0] = c; v3[1] = 0; v3[2] = 0;
-            block_scan3(v3, tot3, scanbuf, bid, tid);
+            block_scan3<NT>(v3, tot3, scanbuf, bid, tid);
         }
         mark(tot3[0] != 2 * n || (LB > 0 && lenb[LB - 1] >= 0x80) || (LB == 0 && n > 0) || misc[1], kStageVarint);
         if (!bad) {
@@ -384,11 +390,11 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 idx++;
             }
         }
-        grp_sync(bid);
+        grp_sync<NT>(bid);
         mark(misc[1] != 0, kStageVarint);
 
         // ---- token scans: positions, literal positions, NEW indices ----
-        const uint32_t tper = (n + kLocThreads - 1) / kLocThreads;
+        const uint32_t tper = (n + NT - 1) / NT;
         const uint32_t i0 = min(n, tid * tper), i1 = min(n, i0 + tper);
         bool any_rep = false;
         {
@@ -407,7 +413,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 }
             if (tbad) misc[1] = 1;
             v3[0] = s_len; v3[1] = s_ll; v3[2] = s_new;
-            block_scan3(v3, tot3, scanbuf, bid, tid);
+            block_scan3<NT>(v3, tot3, scanbuf, bid, tid);
         }
         mark(tot3[0] != R || tot3[1] != n_lit || tot3[2] != n_new || misc[1], kStageTokens);
         if (!bad) {
@@ -428,7 +434,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 lp += ll;
             }
         }
-        any_rep = grp_or(bid, any_rep && !bad);
+        any_rep = grp_or<NT>(bid, any_rep && !bad);
         mark(misc[1] != 0, kStageSources);
 
         // ---- the four-entry history (blocks with repeat codes only) as a
@@ -479,7 +485,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             if (place && (warp > 0 || !any_rep)) {
                 // literal placement: a thread copies a tiny run (<= kLaneBytes)
                 // by itself, all threads at once; eight lanes copy each longer one
-                const int w0 = any_rep ? 1 : 0, nw = kLocWarps - w0;
+                const int w0 = any_rep ? 1 : 0, nw = (NT / 32) - w0;
                 for (uint32_t i = tid - 32 * w0; i < n; i += 32 * nw) {
                     const uint32_t ll = tll[i];
                     if (ll <= kLaneBytes) {
@@ -490,7 +496,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 for (uint32_t i = (warp - w0) * 4 + (lane >> 3); i < n; i += nw * 4)
                     if (tll[i] > kLaneBytes) copy_run8(sout, slit, tlit[i], tpos[i], tll[i], lane & 7);
             }
-            grp_sync(bid);
+            grp_sync<NT>(bid);
             mark(misc[1] != 0, kStageSources);
         }
 
@@ -509,7 +515,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                     dbad = !listed(dl, nd, (uint32_t)a);
             }
             if (dbad) misc[1] = 1;
-            grp_sync(bid);
+            grp_sync<NT>(bid);
             mark(misc[1] != 0, kStageSources);
         }
 
@@ -517,14 +523,14 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             // parse only: one record per token (source, destination offset,
             // match length, command)
             if (!bad)
-                for (uint32_t i = tid; i < n; i += kLocThreads)
+                for (uint32_t i = tid; i < n; i += NT)
                     J.spans[ir.span_base + i] = SpanRec{(uint32_t)tsrc[i], (uint32_t)(tsrc[i] >> 32),
                                                         (uint32_t)(tpos[i] + tll[i]) | ((uint32_t)tml[i] << 16), tcmd[i]};
             if (bad && tid == 0) {
                 set_err_arc(job, a, kErrCorrupt, stage << 24, b);
                 J.npend[ir.slot] = 1;  // per-item status of a parse-only job
             }
-            grp_sync(bid);
+            grp_sync<NT>(bid);
             settle_claim();
             continue;
         }
@@ -535,8 +541,8 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             //      the in-block matches are listed (the literal positions are dead now) ----
             uint16_t* act_list = tlit;
             if (tid == 0) misc[3] = 0;
-            grp_sync(bid);
-            for (uint32_t i = tid; i < n; i += kLocThreads) {
+            grp_sync<NT>(bid);
+            for (uint32_t i = tid; i < n; i += NT) {
                 const uint32_t ml = tml[i];
                 uint8_t st = 0;  // 0: none/done, 1: unresolved in-block, 2: pending
                 if (ml) {
@@ -548,7 +554,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 tstat[i] = st;
                 if (lvl) tlvk[i] = tlvl[i];  // the staging buffer takes the next block's levels below
             }
-            grp_sync(bid);
+            grp_sync<NT>(bid);
             // ---- the stream buffers are free from here on: start the next item's
             //      copies, so that they land while this block finishes ----
             settle_claim();
@@ -557,7 +563,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             // (issued by the last warp, which takes the fewest in-block matches
             // below, so that its loads of the next block's descriptor delay the
             // rounds least)
-            if (tid == kLocThreads - 32) {
+            if (tid == NT - 32) {
                 // in a fused decode, only streams that are already published
                 const bool go = pf_item < job.n_items && (!job.ready || ld_acquire_u32(job.ready + pf_item) != 0);
                 if (go) {
@@ -574,7 +580,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 bool progress = false, left = false;
                 const uint32_t g = lane >> 3, sl = lane & 7;
                 const uint32_t gmask = 0xffu << (8 * g);
-                for (uint32_t base = warp * 4; base < n_act; base += kLocWarps * 4) {
+                for (uint32_t base = warp * 4; base < n_act; base += (NT / 32) * 4) {
                     const uint32_t i = base + g < n_act ? act_list[base + g] : n;
                     const bool act = i < n && tstat[i] == 1;  // the same for the group's lanes
                     uint32_t ml = 0, o = 0, so = 0, d = 1, we = 0;
@@ -615,8 +621,8 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                         progress = true;
                     }
                 }
-                const int any_left = grp_or(bid, left);
-                const int any_prog = grp_or(bid, progress);
+                const int any_left = grp_or<NT>(bid, left);
+                const int any_prog = grp_or<NT>(bid, progress);
                 if (!any_left || !any_prog) break;
             }
             // ---- whatever is still unresolved becomes pending pieces (for a
@@ -631,7 +637,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                     nbytes += tml[i];
                 }
             v3[0] = cnt; v3[1] = nbytes; v3[2] = 0;
-            block_scan3(v3, tot3, scanbuf, bid, tid);
+            block_scan3<NT>(v3, tot3, scanbuf, bid, tid);
             npend = tot3[0];
             pbytes = tot3[1];
             if (lvl) {
@@ -641,11 +647,11 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 // and carry their level, and the level list is built from
                 // them (k_level_fill)
                 const uint32_t Lg = job.n_levels;
-                for (uint32_t l = tid; l <= Lg; l += kLocThreads) lhist[l] = 0;
-                grp_sync(bid);
+                for (uint32_t l = tid; l <= Lg; l += NT) lhist[l] = 0;
+                grp_sync<NT>(bid);
                 for (uint32_t i = i0; i < i1; i++)
                     if (tstat[i]) atomicAdd(&lhist[min(max((uint32_t)tlvk[i], 1u), Lg)], pieces_of(tml[i]));
-                grp_sync(bid);
+                grp_sync<NT>(bid);
                 if (warp == 0) {
                     uint32_t carry = 0;
                     uint32_t* row = job.lvl_tab + (uint64_t)ir.slot * (Lg + 1);
@@ -672,19 +678,19 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 }
             }
         }
-        grp_sync(bid);
+        grp_sync<NT>(bid);
         if (bad) {
             if (tid == 0) set_err_arc(job, a, kErrCorrupt, stage << 24, b);
             npend = 0;
             if (lvl)  // an empty row: the level rounds take nothing from this block
-                for (uint32_t l = tid; l <= job.n_levels; l += kLocThreads)
+                for (uint32_t l = tid; l <= job.n_levels; l += NT)
                     job.lvl_tab[(uint64_t)ir.slot * (job.n_levels + 1) + l] = 0;
         }
         // ---- write the block (pending bytes are filled by the cross-block pass) ----
         uint8_t* gout = J.out + (uint64_t)ir.slot * kBlock;
         const uint32_t nv = R / 16;
-        for (uint32_t i = tid; i < nv; i += kLocThreads) reinterpret_cast<uint4*>(gout)[i] = reinterpret_cast<uint4*>(sout)[i];
-        for (uint32_t x = 16 * nv + tid; x < R; x += kLocThreads) gout[x] = sout[x];
+        for (uint32_t i = tid; i < nv; i += NT) reinterpret_cast<uint4*>(gout)[i] = reinterpret_cast<uint4*>(sout)[i];
+        for (uint32_t x = 16 * nv + tid; x < R; x += NT) gout[x] = sout[x];
         {
             // the pending bitmap is written for every block (all clear when nothing
             // is pending, a corrupt block included), so readers need no second
@@ -692,7 +698,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             uint4* gp = reinterpret_cast<uint4*>(J.pmap + (uint64_t)ir.slot * (kBlock / 32));
             const uint4* sp = reinterpret_cast<const uint4*>(pend);
             const uint4* np4 = reinterpret_cast<const uint4*>(need);
-            for (uint32_t i = tid; i < kBlock / 128; i += kLocThreads) {
+            for (uint32_t i = tid; i < kBlock / 128; i += NT) {
                 uint4 v = npend ? sp[i] : make_uint4(0, 0, 0, 0);
                 if (partial) {  // unwanted bytes are never read: leave them out of the bitmap
                     const uint4 m = np4[i];
@@ -708,7 +714,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 atomicAdd(reinterpret_cast<unsigned long long*>(job.counters + kStatPendBytes), (unsigned long long)pbytes);
             }
         }
-        grp_sync(bid);
+        grp_sync<NT>(bid);
         settle_claim();
     }
 }

@@ -60,7 +60,7 @@ namespace {
 // Plan summary written by k_plan_small and read back by the host.
 struct NaSummary {
     int32_t status;       // 0 ok, -2 corrupt, -1 beyond the static limits
-    uint32_t n_blocks, min_match, max_tok, max_lenb, has_deps;
+    uint32_t n_blocks, min_match, max_tok, max_lenb, max_lit, has_deps;
     uint64_t total, span_slots, stream_bytes;
 };
 static_assert(sizeof(NaSummary) <= 64, "summary");
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(256) k_plan_small(const uint8_t* a, uint64_t l
     if (tid == 0) {
         int st = bad;
         uint64_t scratch = 0, slots = 0;
-        uint32_t max_tok = 1, max_lenb = 1;
+        uint32_t max_tok = 1, max_lenb = 1, max_lit = 0;
         for (uint32_t b = 0; b < nb && !st; b++) {
             BlockDev& bd = blk[b];
             const uint64_t sz = bd.scratch;
@@ -210,6 +210,7 @@ __global__ void __launch_bounds__(256) k_plan_small(const uint8_t* a, uint64_t l
             slots += bd.n_tok + kSpanSlack;
             max_tok = max(max_tok, bd.n_tok);
             max_lenb = max(max_lenb, bd.s_raw[kLen]);
+            max_lit = max(max_lit, bd.s_raw[kLit]);
         }
         if (!st && (scratch + 64 > kNaStreamBytes || slots > kNaSpanSlots)) st = -1;
         S->status = st;
@@ -217,6 +218,7 @@ __global__ void __launch_bounds__(256) k_plan_small(const uint8_t* a, uint64_t l
         S->min_match = min_match;
         S->max_tok = max_tok;
         S->max_lenb = max_lenb;
+        S->max_lit = max_lit;
         S->total = total;
         S->has_deps = off_deps != 0;
         S->span_slots = slots;
@@ -261,7 +263,7 @@ extern "C" int aceapex_decode_noalloc(const void* d_arc, uint64_t arc_len, void*
     if (S.status != 0) return ACEAPEX_E_CORRUPT;
     if (out_cap < S.total) return ACEAPEX_E_ARG;
     if (S.n_blocks == 0) return ACEAPEX_OK;
-    const size_t lsm = local_smem_bytes(S.max_tok, S.max_lenb);
+    const size_t lsm = local_smem_bytes(S.max_tok, S.max_lenb, S.max_lit);
     if (lsm > 227 * 1024) return ACEAPEX_E_CORRUPT;  // as the regular plan: no valid block needs that much
     JobDev job{};
     ArcJob& J = job.one;
@@ -286,6 +288,7 @@ extern "C" int aceapex_decode_noalloc(const void* d_arc, uint64_t arc_len, void*
     job.timeout_ns = 2000000000ull;
     job.max_tok = S.max_tok;
     job.max_lenb = S.max_lenb;
+    job.max_lit = S.max_lit;
     job.lists[0] = reinterpret_cast<JobDev::ListEnt*>(base + kOffLists);
     job.lists[1] = job.lists[0] + kNaSpanSlots;
     int n_sms = 0;

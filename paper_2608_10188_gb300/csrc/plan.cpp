@@ -67,6 +67,7 @@ int build_plan(const uint8_t* a, uint64_t len, Plan* P, std::string* why) {
     P->deps.clear();
     P->max_tok = 1;
     P->max_lenb = 1;
+    P->max_lit = 0;
     P->max_level = 0;
     P->tokens = 0;
     uint64_t scratch = 0;
@@ -144,6 +145,7 @@ int build_plan(const uint8_t* a, uint64_t len, Plan* P, std::string* why) {
         scratch += soff;
         if (n_tok > P->max_tok) P->max_tok = n_tok;
         if (bd.s_raw[kLen] > P->max_lenb) P->max_lenb = bd.s_raw[kLen];
+        if (bd.s_raw[kLit] > P->max_lit) P->max_lit = bd.s_raw[kLit];
         P->tokens += n_tok;
         if (P->span_slots >= (1ull << 32)) return fail("too many tokens");
     }

@@ -11,7 +11,7 @@ namespace acx {
 
 struct Plan {
     uint64_t total = 0, archive_bytes = 0, tokens = 0, scratch_bytes = 0, span_slots = 0;
-    uint32_t n_blocks = 0, flags = 0, min_match = 0, max_tok = 0, max_lenb = 0;
+    uint32_t n_blocks = 0, flags = 0, min_match = 0, max_tok = 0, max_lenb = 0, max_lit = 0;
     uint16_t freq[4][256];
     bool table_ok[4];
     std::vector<uint32_t> dtab;   // 4 x 4096 decode entries

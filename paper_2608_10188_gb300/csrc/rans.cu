@@ -95,9 +95,10 @@ static std::atomic<int> g_sm_count{0};
 
 void note_sm_count(int n_sms) { g_sm_count.store(n_sms); }
 
+int noted_sm_count() { return std::max(g_sm_count.load(), 1); }
+
 int job_grid(int full, uint64_t need) {
-    const int n_sms = std::max(g_sm_count.load(), 1);
-    const uint64_t g = std::max<uint64_t>(need, (uint64_t)n_sms);
+    const uint64_t g = std::max<uint64_t>(need, (uint64_t)noted_sm_count());
     return (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)full, g));
 }
 

@@ -518,11 +518,12 @@ bool aceapex_server::form_tick(int li) {
         job.timeout_ns = (uint64_t)c->params.timeout_us * 1000ull;
         job.max_tok = S.max_tok;
         job.max_lenb = S.max_lenb;
+        job.max_lit = S.max_lit;
         job.flags = need.empty() ? 0 : kJobNeed;
         job.lists[0] = (JobDev::ListEnt*)lists.p;
         job.lists[1] = job.lists[0] + std::max<uint64_t>(S.span_slots, 1);
         LaunchPlan lp;
-        rc = launch_plan(c, c->params, S.max_tok, S.max_lenb, &lp, job.flags);
+        rc = launch_plan(c, c->params, S.max_tok, S.max_lenb, S.max_lit, &lp, job.flags);
         // the cross-block pass of a tick holds a 1024-thread CTA per 32 blocks
         // at most, so that ticks on other lanes find SMs beside it
         lp.grid_ext = std::min<int>(lp.grid_ext, (int)std::max<size_t>(1, (nblk + 31) / 32));

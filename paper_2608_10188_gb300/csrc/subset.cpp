@@ -58,6 +58,7 @@ void acx::subset_plan(const Plan& P, const uint32_t* blocks, const uint32_t* slo
     S->span_slots = 0;
     S->max_tok = 1;
     S->max_lenb = 1;
+    S->max_lit = 0;
     for (size_t i = 0; i < n; i++) {
         const BlockDev& bd = P.blk[blocks[i]];
         ItemDev& it = S->items[i];
@@ -70,6 +71,7 @@ void acx::subset_plan(const Plan& P, const uint32_t* blocks, const uint32_t* slo
         S->span_slots += bd.n_tok + kSpanSlack;
         S->max_tok = std::max(S->max_tok, bd.n_tok);
         S->max_lenb = std::max(S->max_lenb, bd.s_raw[kLen]);
+        S->max_lit = std::max(S->max_lit, bd.s_raw[kLit]);
     }
     S->scratch_bytes += 64;
 }
@@ -171,11 +173,12 @@ extern "C" int aceapex_decode_range(aceapex_ctx* c, aceapex_archive* A, uint64_t
     job.timeout_ns = (uint64_t)c->params.timeout_us * 1000ull;
     job.max_tok = S.max_tok;
     job.max_lenb = S.max_lenb;
+    job.max_lit = S.max_lit;
     job.lists[0] = (JobDev::ListEnt*)c->lists.p;
     job.lists[1] = job.lists[0] + S.span_slots;
     job.flags = flags;
     LaunchPlan lp;
-    if ((rc = launch_plan(c, c->params, S.max_tok, S.max_lenb, &lp, flags))) return rc;
+    if ((rc = launch_plan(c, c->params, S.max_tok, S.max_lenb, S.max_lit, &lp, flags))) return rc;
     if ((rc = enqueue_job(c, job, lp, 4, nullptr, 0, st, stats ? c->ev : nullptr))) return rc;
     const GatherReq req{(uint8_t*)d_out, start, len};
     if ((e = launch_gather(&req, nullptr, 1, len, J.out, A->d_slot, st)) != cudaSuccess)
