@@ -147,6 +147,7 @@ struct JobDev {
     uint32_t max_lenb;
     uint32_t max_lit;
     uint32_t flags;           // kJob* bits
+    uint32_t rans_parts;      // tickets per work item of the entropy stage (set at its launch)
     uint32_t chunk;           // work items per ticket of the entropy stage and the local pass (0 = 1)
     uint32_t wait_ns;         // cross-block round 0: how long a piece may wait for its sources before it
                               // is left to the later rounds (0xffffffff: until the deadline)

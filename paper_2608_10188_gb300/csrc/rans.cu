@@ -56,34 +56,43 @@ __global__ void __launch_bounds__(kRansWarps * 32) k_rans(JobDev job) {
             __syncthreads();
             if (threadIdx.x == 0) S.arc = a;
         }
-        const uint32_t n_a = J.hi - J.lo;
+        // tickets: the blocks, or (rans_parts) their literals, then their other
+        // parts; a lone archive's first run of every warp is its own, so that
+        // the work starts spread over the SMs however their CTAs come up
+        const uint32_t n_blk = J.hi - J.lo, n_a = n_blk * job.rans_parts;
         const uint32_t chunk = job.chunk ? job.chunk : 1u;
-        uint32_t cnext = 0, cleft = 0;  // this warp's current run of `chunk` tickets
+        const uint32_t own = job.n_arcs == 1 ? gridDim.x * kRansWarps * chunk : 0u;
+        uint32_t cnext = (warp * gridDim.x + blockIdx.x) * chunk;  // this warp's current run of `chunk` tickets
+        uint32_t cleft = own ? chunk : 0u;
         for (;;) {
             if (cleft == 0) {
                 uint32_t t0 = 0;
                 if (lane == 0) t0 = atomicAdd(&tickets[a], chunk);
-                cnext = __shfl_sync(ACX_FULL, t0, 0);
+                cnext = own + __shfl_sync(ACX_FULL, t0, 0);
                 cleft = chunk;
             }
             const uint32_t tk = cnext++;
             cleft--;
             if (tk >= n_a) break;
-            rans_block(job, a, J, item_ref(J, J.order ? J.order[tk] : tk), smem_u32(&S.tab[0][0]), ring_s,
+            const uint32_t turn = tk / n_blk, i = tk - turn * n_blk;
+            const uint32_t part = job.rans_parts == 1 ? kRansAll : kRansParts - 1 - turn;
+            rans_block(job, a, J, item_ref(J, J.order ? J.order[i] : i), part, smem_u32(&S.tab[0][0]), ring_s,
                        smem_u32(&S.stage[warp][0]), &S.bar[warp][0], &S.sbar[warp], seq, sphase, lane, deadline);
         }
+        if (job.n_arcs == 1) break;
         __syncthreads();
-        if (threadIdx.x == 0) {
-            int best = -1;
-            uint32_t best_left = 0;
-            for (uint32_t k = 0; k < job.n_arcs; k++) {
-                const ArcJob Jk = load_arc(job, (int)k);
+        if (warp == 0) {
+            // the archive with the most tickets left, the lowest of equals
+            uint32_t best = 0xffffffffu, best_left = 0;
+            for (uint32_t k = lane; k < job.n_arcs; k += 32) {
                 const uint32_t taken = *((volatile uint32_t*)&tickets[k]);
-                const uint32_t n_k = Jk.hi - Jk.lo;
+                const uint32_t n_k = (job.arcs[k].hi - job.arcs[k].lo) * job.rans_parts;
                 const uint32_t left = taken < n_k ? n_k - taken : 0;
-                if (left > best_left) { best_left = left; best = (int)k; }
+                if (left > best_left) { best_left = left; best = k; }
             }
-            S.next_arc = best;
+            const uint32_t most = __reduce_max_sync(ACX_FULL, best_left);
+            best = __reduce_min_sync(ACX_FULL, best_left == most ? best : 0xffffffffu);
+            if (lane == 0) S.next_arc = most ? (int)best : -1;
         }
         __syncthreads();
     }
@@ -107,13 +116,23 @@ cudaError_t launch_prologue(uint32_t* counters, uint32_t n_counters, cudaStream_
     return cudaGetLastError();
 }
 
-cudaError_t launch_rans(const JobDev& job, int grid, cudaStream_t st) {
+cudaError_t launch_rans(const JobDev& job_in, int grid, cudaStream_t st) {
+    JobDev job = job_in;
     const size_t sm = rans_smem_bytes();
     cudaError_t e = cudaFuncSetAttribute(k_rans, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    // a small job needs no more CTAs than its warps can take ticket runs
+    // When every part of every block finds a warp at once, a block's streams
+    // decode on three warps and only the longest counts (one 10 KB text block
+    // 47 -> 27 us, 4 MiB of text 62 -> 31, 4 MiB DNA-like 65 -> 54); with more
+    // blocks the warps are busy anyway, and a part would only cost a ticket.
+    const uint64_t warps = (uint64_t)kRansWarps * (uint64_t)grid;
+    job.rans_parts = (uint64_t)job.n_items * kRansParts <= warps ? kRansParts : 1;
+    // One CTA per SM while that gives every ticket run a warp (each CTA loads
+    // the 64 KiB of tables), else all: with a grid cut to the need, some SMs
+    // have twice the warps of others (4,097 blocks: 95 us, 90 with all).
     const uint64_t per_cta = (uint64_t)kRansWarps * (job.chunk ? job.chunk : 1);
-    grid = job_grid(grid, (job.n_items + per_cta - 1) / per_cta);
+    const uint64_t need = ((uint64_t)job.n_items * job.rans_parts + per_cta - 1) / per_cta;
+    if (need <= (uint64_t)noted_sm_count()) grid = std::min(grid, noted_sm_count());
     k_rans<<<grid, kRansWarps * 32, sm, st>>>(job);
     return cudaGetLastError();
 }

@@ -14,7 +14,7 @@
 //    by 512-byte 1-D TMA bulk copies (cp.async.bulk + mbarrier), kept up to
 //    three chunks ahead of the decoder;
 //  * K = 64 / 128 lanes run as 2 / 4 independent states per warp lane (ILP);
-//  * ring residency is checked once per 8 steps (of 32 symbols), not per step;
+//  * ring residency is checked once per 16 steps (of 32 symbols), not per step;
 //  * the tables and rings are read at 32-bit shared-window addresses, and the
 //    renormalisation is branch-free (every lane reads its candidate word).
 // Every wait is bounded by %globaltimer.
@@ -224,24 +224,43 @@ static __device__ __noinline__ bool rans_stream4(uint32_t tab_s, const uint8_t* 
     return rans_stream<4>(tab_s, body, enc, n, K, out, ring_s, stage_s, bar, seq, lane, deadline);
 }
 
-// The short streams of a block (cmd, len, off) decoded concurrently by one
+// Which of a block's short streams (cmd, len, off) decode side by side on one
+// warp: in that order, each one that still fits the 32 lanes and whose words
+// fit the ring; fewer than two are not worth it.  A genome block's three fit
+// together; of a text block, whose offsets take all lanes, the commands and
+// lengths (8 and 16 lanes, 106 steps each) run as one (200 MiB of text: 247 ->
+// 203 us for the stage).
+__device__ __forceinline__ uint32_t short_group(const BlockDev& bd) {
+    uint32_t lanes = 0, bytes = 0, mask = 0;
+#pragma unroll
+    for (int g = 0; g < 3; g++) {
+        const uint32_t K = bd.s_K[g], hdr = (4 * K + 15) & ~15u, enc = bd.s_enc[g];
+        if (!bd.s_raw[g] || !(bd.rans_mask & (1u << g)) || enc < hdr) continue;
+        const uint32_t nw = (enc - hdr + 15) & ~15u;
+        if (lanes + K > 32 || bytes + nw > 2 * kRingWords) continue;
+        lanes += K;
+        bytes += nw;
+        mask |= 1u << g;
+    }
+    return __popc(mask) >= 2 ? mask : 0;
+}
+
+// The short streams of `mask` (see short_group) decoded concurrently by one
 // warp: stream g runs on lanes [lo_g, lo_g + K_g) with its own word pointer;
-// their words are staged whole into the warp's ring by TMA.  Returns 0 on
-// success, 1 when the layout does not fit (caller decodes them one by one),
-// -1 on a format violation or an expired wait.
-__device__ __forceinline__ int rans_short3(uint32_t tab0_s, const BlockDev& bd, const uint8_t* pay, uint8_t* scr,
-                                           uint32_t ring_s, uint64_t* sbar, uint32_t& sphase, int lane,
+// their words are staged whole into the warp's ring by TMA.  Returns false on
+// a format violation or an expired wait.
+__device__ __forceinline__ bool rans_short(uint32_t mask, uint32_t tab0_s, const BlockDev& bd, const uint8_t* pay,
+                                           uint8_t* scr, uint32_t ring_s, uint64_t* sbar, uint32_t& sphase, int lane,
                                            uint64_t deadline) {
     uint32_t lo[3], K[3], W[3], hdr[3], roff[3], nw_bytes[3];
     uint32_t lanes = 0, bytes = 0;
     for (int g = 0; g < 3; g++) {
         K[g] = 0;
-        if (!bd.s_raw[g] || !(bd.rans_mask & (1u << g))) continue;
+        if (!(mask & (1u << g))) continue;
         K[g] = bd.s_K[g];
-        if (K[g] > 32) return 1;
         hdr[g] = (4 * K[g] + 15) & ~15u;
         const uint32_t enc = bd.s_enc[g];
-        if (enc < hdr[g] || ((enc - hdr[g]) & 1)) return -1;
+        if (enc < hdr[g] || ((enc - hdr[g]) & 1)) return false;
         W[g] = (enc - hdr[g]) >> 1;
         nw_bytes[g] = (2 * W[g] + 15) & ~15u;
         lo[g] = lanes;
@@ -249,8 +268,6 @@ __device__ __forceinline__ int rans_short3(uint32_t tab0_s, const BlockDev& bd, 
         roff[g] = bytes;
         bytes += nw_bytes[g];
     }
-    if (lanes > 32 || bytes > 2 * kRingWords) return 1;
-    if (lanes == 0) return 0;
     // stage every short stream's words
     __syncwarp();
     if (lane == 0) {
@@ -285,7 +302,7 @@ __device__ __forceinline__ int rans_short3(uint32_t tab0_s, const BlockDev& bd, 
         while (!mbar_try_wait(sbar, sphase & 1))
             if ((++spins & 1023) == 0 && gtimer() > deadline) { w = false; break; }
         sphase++;
-        if (!__all_sync(ACX_FULL, w)) return -1;
+        if (!__all_sync(ACX_FULL, w)) return false;
     }
     ok = __all_sync(ACX_FULL, ok);
     const uint32_t lt_mask = (1u << lane) - 1;
@@ -317,7 +334,7 @@ __device__ __forceinline__ int rans_short3(uint32_t tab0_s, const BlockDev& bd, 
     ok = __all_sync(ACX_FULL, ok);
     const bool fin = my < 0 || (p == Wg && x == kL);
     __syncwarp();  // the ring is free again for the next stream's copies
-    return __all_sync(ACX_FULL, ok && fin) ? 0 : -1;
+    return __all_sync(ACX_FULL, ok && fin);
 }
 
 __device__ __forceinline__ void copy_stored(const uint8_t* __restrict__ src, uint8_t* __restrict__ dst, uint32_t n, int lane) {
@@ -327,29 +344,41 @@ __device__ __forceinline__ void copy_stored(const uint8_t* __restrict__ src, uin
     for (uint32_t i = lane; i < nv; i += 32) d[i] = s[i];
 }
 
-// Entropy-decode one work item's streams (one warp) into its decoded-stream
-// scratch: the three short streams together when they fit the warp, then the
-// rest one by one (the literal stream is skipped by a parse-only job).
-// tab0_s is the shared address of the four decode tables; bar (kSlots
-// barriers), sbar, the ring and the symbol stage (kStageBytes, 16-aligned)
-// are the warp's own.  A corrupt stream sets the
-// job's (and the archive's) error status.
+// Parts of a block's entropy decode that warps may take one by one: 0 = the
+// commands and lengths (with the offsets when they decode side by side), 1 =
+// the offsets otherwise, 2 = the literals; kRansAll = the whole block.
+constexpr uint32_t kRansParts = 3, kRansAll = 3;
+
+// Entropy-decode one work item's streams, or one part of them (one warp), into
+// its decoded-stream scratch: the short streams that fit the warp together
+// side by side, then the rest one by one (the literal stream is skipped by a
+// parse-only job).  tab0_s is the shared address of the four decode tables;
+// bar (kSlots barriers), sbar, the ring and the symbol stage (kStageBytes,
+// 16-aligned) are the warp's own.  A corrupt stream sets the job's (and the
+// archive's) error status.
 __device__ __forceinline__ void rans_block(const JobDev& job, int a, const ArcJob& J, const ItemRef& ir,
-                                           uint32_t tab0_s, uint32_t ring_s, uint32_t stage_s, uint64_t* bar,
-                                           uint64_t* sbar, uint32_t& seq, uint32_t& sphase, int lane,
+                                           uint32_t part, uint32_t tab0_s, uint32_t ring_s, uint32_t stage_s,
+                                           uint64_t* bar, uint64_t* sbar, uint32_t& seq, uint32_t& sphase, int lane,
                                            uint64_t deadline) {
     const uint32_t b = ir.blk;
     if (J.items && J.slot && lane == 0) J.slot[b] = ir.slot;  // read by the cross-block pass
     const BlockDev& bd = J.blk[b];
     const uint8_t* pay = J.arc + bd.payload;
     uint8_t* scr = J.scratch + ir.scratch;
+    const uint32_t together = short_group(bd);
+    // the part's streams (a parse needs no literals)
+    uint32_t mask = (job.flags & kJobIndex) ? 7u : 15u;
+    if (part == 0) mask &= 3u | together;
+    if (part == 1) mask &= 4u & ~together;
+    if (part == 2) mask &= 8u;
     bool ok = true;
     int fs = 0;
-    const int sh = rans_short3(tab0_s, bd, pay, scr, ring_s, sbar, sphase, lane, deadline);
-    if (sh < 0) ok = false;
-    const int n_streams = (job.flags & kJobIndex) ? 3 : 4;  // a parse needs no literals
-    for (int s = 0; s < n_streams && ok; s++) {
-        if (sh == 0 && s < 3 && (bd.rans_mask & (1u << s))) continue;  // decoded above
+    if (together && part != 1 && part != 2) {
+        ok = rans_short(together, tab0_s, bd, pay, scr, ring_s, sbar, sphase, lane, deadline);
+        mask &= ~together;
+    }
+    for (int s = 0; s < 4 && ok; s++) {
+        if (!(mask & (1u << s))) continue;
         fs = s;
         const uint32_t n = bd.s_raw[s];
         if (n == 0) continue;
