@@ -81,35 +81,39 @@ __device__ __forceinline__ int grp_or(uint32_t bid, int v) {
     return (int)r;
 }
 
-// Group-wide exclusive scan of three u32 values per thread (tid: the thread
-// in its group).
-template <int NT>
-__device__ __forceinline__ void block_scan3(uint32_t v[3], uint32_t tot[3], uint32_t* buf, uint32_t bid, int tid) {
+// Group-wide exclusive scan of V u32 values per thread (tid: the thread in
+// its group).
+template <int NT, int V>
+__device__ __forceinline__ void block_scan(uint32_t (&v)[V], uint32_t (&tot)[V], uint32_t* buf, uint32_t bid, int tid) {
     const int lane = tid & 31, warp = tid >> 5;
-    uint32_t inc[3] = {v[0], v[1], v[2]};
+    uint32_t inc[V];
+#pragma unroll
+    for (int k = 0; k < V; k++) inc[k] = v[k];
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
 #pragma unroll
-        for (int k = 0; k < 3; k++) {
+        for (int k = 0; k < V; k++) {
             const uint32_t y = __shfl_up_sync(ACX_FULL, inc[k], o);
             if (lane >= o) inc[k] += y;
         }
     }
     if (lane == 31)
-        for (int k = 0; k < 3; k++) buf[warp * 3 + k] = inc[k];
+        for (int k = 0; k < V; k++) buf[warp * V + k] = inc[k];
     grp_sync<NT>(bid);
-    uint32_t wpre[3] = {0, 0, 0}, t[3] = {0, 0, 0};
+    uint32_t wpre[V], t[V];
 #pragma unroll
-    for (int w = 0; w < (NT / 32); w++) {
+    for (int k = 0; k < V; k++) wpre[k] = t[k] = 0;
 #pragma unroll
-        for (int k = 0; k < 3; k++) {
-            const uint32_t s = buf[w * 3 + k];
+    for (int w = 0; w < NT / 32; w++) {
+#pragma unroll
+        for (int k = 0; k < V; k++) {
+            const uint32_t s = buf[w * V + k];
             if (w < warp) wpre[k] += s;
             t[k] += s;
         }
     }
 #pragma unroll
-    for (int k = 0; k < 3; k++) {
+    for (int k = 0; k < V; k++) {
         v[k] = wpre[k] + inc[k] - v[k];
         tot[k] = t[k];
     }
@@ -194,6 +198,129 @@ __device__ __forceinline__ void copy_run8(uint8_t* sout, const uint8_t* lit, uin
         reinterpret_cast<uint4*>(sout)[q] = make_uint4(__funnelshift_r(x0, x1, sh), __funnelshift_r(x1, x2, sh),
                                                        __funnelshift_r(x2, x3, sh), __funnelshift_r(x3, x4, sh));
     }
+}
+
+// Copy out[o, o + ml) = out[so, so + ml) (disjoint), by one thread: bytes up to
+// a word boundary of the destination, words from two source words each, four
+// at a time, bytes at the end.  Words may reach 3 bytes past the source run
+// (never past the block: a source ends at or before its destination).
+__device__ __forceinline__ void copy_lane(uint8_t* out, uint32_t so, uint32_t o, uint32_t ml) {
+    const uint32_t e = o + ml, q0 = (o + 3) >> 2, q1 = e >> 2;
+    const uint32_t head = min(4 * q0, e), tail = max(4 * q1, head);
+    for (uint32_t x = o; x < head; x++) out[x] = out[so + x - o];
+    const uint32_t* lw = reinterpret_cast<const uint32_t*>(out);
+    uint32_t* ow = reinterpret_cast<uint32_t*>(out);
+    const uint32_t s0 = so + 4 * q0 - o, sh = 8 * (s0 & 3), w = s0 >> 2;
+    for (uint32_t q = q0; q < q1; q += 4) {
+        uint32_t x[5];
+#pragma unroll
+        for (int u = 0; u < 5; u++) x[u] = q + u <= q1 ? lw[w + (q - q0) + u] : 0;
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (q + u < q1) ow[q + u] = __funnelshift_r(x[u], x[u + 1], sh);
+    }
+    for (uint32_t x = tail; x < e; x++) out[x] = out[so + x - o];
+}
+
+// Periodic fill out[o + k] = out[so + (k mod d)], k < ml, d < ml, by the eight
+// lanes sl of a lane group: it reads the period window [so, so + d) only, so
+// the lanes are independent; whole destination words as one store each.
+__device__ __forceinline__ void fill_run8(uint8_t* out, uint32_t so, uint32_t o, uint32_t ml, uint32_t d, uint32_t sl) {
+    const uint32_t e = o + ml, q0 = (o + 3) >> 2, q1 = e >> 2;  // whole words [q0, q1)
+    // ragged ends of at most 3 bytes: lanes 0..3 the head, 4..7 the tail
+    const uint32_t edge = sl < 4 ? o + sl : max(4 * q1, 4 * q0) + sl - 4, edge_end = sl < 4 ? min(4 * q0, e) : e;
+    if (edge < edge_end) out[edge] = out[so + (edge - o) % d];
+    uint32_t r = (4 * (q0 + sl) - o) % d;
+    const uint32_t step = 32 % d;
+    for (uint32_t q = q0 + sl; q < q1; q += 8) {
+        uint32_t v = 0, x = r;
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            v |= (uint32_t)out[so + x] << (8 * u);
+            if (++x == d) x = 0;
+        }
+        reinterpret_cast<uint32_t*>(out)[q] = v;
+        r += step;
+        if (r >= d) r -= d;
+    }
+}
+
+// One pass by one warp over the listed in-block matches act[first + k],
+// act[first + stride + k], .., with 32 / G matches at a time (k < 32 / G) and
+// G lanes a match.  A match whose source window has no pending byte is filled,
+// its bits are cleared and its status becomes 0.  Returns, over the lane's
+// matches, bit 0: one is left; bit 1: one was filled.
+//
+// G = 8 suits blocks of some tens of matches, whose copies are then short; a
+// block with hundreds (the first blocks of a text, which hold no earlier
+// blocks to copy from) is bound by its number of passes, and G = 1 looks after
+// eight times as many in each: a lane copies a short plain match, eight lanes
+// each longer or periodic one (one 10 KB text block 35 -> 23 us in the local
+// pass, 4 MiB of text 60 -> 42, 64 MiB in 8 MiB segments 189 -> 164).  Groups of 128
+// threads, whose blocks have few tokens, go without it: the code alone costs
+// them (254 MB genome 318 -> 332 us; with G = 1 at every size 411).
+constexpr uint32_t kLaneCopy = 64;
+constexpr uint32_t kManyMatches = 64;  // more: G = 1
+template <uint32_t G>
+__device__ __forceinline__ uint32_t match_pass(const uint16_t* act, uint32_t n_act, uint32_t first, uint32_t stride,
+                                               uint8_t* sout, uint32_t* pend, uint8_t* tstat, const uint16_t* tml,
+                                               const uint16_t* tpos, const uint16_t* tll, const uint64_t* tsrc,
+                                               uint64_t B, int lane) {
+    uint32_t res = 0;
+    const uint32_t g = lane / G, sl = lane % G, gmask = (G == 8 ? 0xffu : 1u) << (G * g);
+    for (uint32_t base = first; base < n_act; base += stride) {
+        const uint32_t i = base + g < n_act ? act[base + g] : 0;
+        const bool on = base + g < n_act && tstat[i] == 1;  // the same for the group's lanes
+        uint32_t ml = 0, o = 0, so = 0, d = 1, we = 0;
+        bool busy = false;
+        if (on) {
+            ml = tml[i];
+            o = tpos[i] + tll[i];
+            so = (uint32_t)(tsrc[i] - B);
+            d = o - so;
+            we = so + min(d, ml);  // periodic source window [so, we)
+            for (uint32_t w = (so >> 5) + sl; w <= ((we - 1) >> 5); w += G)
+                busy |= (((volatile uint32_t*)pend)[w] & range_mask(w, so, we)) != 0;
+        }
+        const uint32_t bm = __ballot_sync(ACX_FULL, busy);  // every lane, active or not
+        const bool ready = on && (bm & gmask) == 0;
+        if (on && !ready) res |= 1;
+        __threadfence_block();  // source reads after the readiness reads
+        if (G == 8) {
+            if (ready) {
+                if (d >= ml) copy_run8(sout, sout, so, o, ml, sl);
+                else fill_run8(sout, so, o, ml, d, sl);
+            }
+        } else {
+            const bool mine = ready && d >= ml && ml <= kLaneCopy;
+            if (mine) copy_lane(sout, so, o, ml);
+            uint32_t rest = __ballot_sync(ACX_FULL, ready && !mine);
+            while (rest) {
+                uint32_t k = 32;  // the next four, eight lanes each
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    if (lane >> 3 == u && rest) k = __ffs(rest) - 1;
+                    rest &= rest - 1;  // (0 stays 0)
+                }
+                const uint32_t ml2 = __shfl_sync(ACX_FULL, ml, k & 31), o2 = __shfl_sync(ACX_FULL, o, k & 31),
+                               so2 = __shfl_sync(ACX_FULL, so, k & 31);
+                if (k < 32) {
+                    if (o2 - so2 >= ml2) copy_run8(sout, sout, so2, o2, ml2, lane & 7);
+                    else fill_run8(sout, so2, o2, ml2, o2 - so2, lane & 7);
+                }
+            }
+        }
+        __syncwarp();
+        __threadfence_block();
+        if (ready) {
+            for (uint32_t w = (o >> 5) + sl; w <= ((o + ml - 1) >> 5); w += G)
+                atomicAnd(&pend[w], ~range_mask(w, o, o + ml));
+            if (sl == 0) tstat[i] = 0;
+            res |= 2;
+        }
+        __syncwarp();
+    }
+    return res;
 }
 
 // Issue the 1-D TMA copies of an item's four decoded streams (16-aligned,
@@ -327,7 +454,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
         //      they were prefetched during the previous block) ----
         if (!bad && tid == 0 && !prefetched && (!job.ready || wait_ready(job.ready, item, deadline)))
             stage_streams(job, item, tcmd, lenb, soff, slit, tlvl, bar);
-        for (uint32_t i = tid; i < kBlock / 32; i += NT) pend[i] = 0;
+        for (uint32_t i = tid; i < kBlock / 128; i += NT) reinterpret_cast<uint4*>(pend)[i] = make_uint4(0, 0, 0, 0);
         if (tid == 0) misc[1] = 0;
         // wanted bytes of this item (all when it names none)
         const bool partial = (job.flags & kJobNeed) && ir.need_n != 0;
@@ -356,7 +483,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
         }
 
         // ---- varints: each byte < 0x80 ends a value ----
-        uint32_t v3[3], tot3[3];
+        uint32_t v1[1], tot1[1], v3[3], tot3[3], v2[2], tot2[2];
         const uint32_t per = (LB + NT - 1) / NT;
         const uint32_t j0 = min(LB, tid * per), j1 = min(LB, j0 + per);
         {
@@ -370,12 +497,12 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                     if (by >= 0x80 && j >= 2 && lenb[j - 1] >= 0x80 && lenb[j - 2] >= 0x80) vbad = true;
                 }
             if (vbad) misc[1] = 1;
-            v3[0] = c; v3[1] = 0; v3[2] = 0;
-            block_scan3<NT>(v3, tot3, scanbuf, bid, tid);
+            v1[0] = c;
+            block_scan<NT, 1>(v1, tot1, scanbuf, bid, tid);
         }
-        mark(tot3[0] != 2 * n || (LB > 0 && lenb[LB - 1] >= 0x80) || (LB == 0 && n > 0) || misc[1], kStageVarint);
+        mark(tot1[0] != 2 * n || (LB > 0 && lenb[LB - 1] >= 0x80) || (LB == 0 && n > 0) || misc[1], kStageVarint);
         if (!bad) {
-            uint32_t idx = v3[0];
+            uint32_t idx = v1[0];
             for (uint32_t j = j0; j < j1; j++) {
                 const uint8_t by = lenb[j];
                 if (by >= 0x80) continue;
@@ -413,7 +540,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 }
             if (tbad) misc[1] = 1;
             v3[0] = s_len; v3[1] = s_ll; v3[2] = s_new;
-            block_scan3<NT>(v3, tot3, scanbuf, bid, tid);
+            block_scan<NT, 3>(v3, tot3, scanbuf, bid, tid);
         }
         mark(tot3[0] != R || tot3[1] != n_lit || tot3[2] != n_new || misc[1], kStageTokens);
         if (!bad) {
@@ -572,57 +699,15 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 }
                 misc[2] = go;
             }
-            // ---- in-block matches: rounds of ready periodic fills over the
-            //      listed matches; each warp works on four matches at once,
-            //      eight lanes per match ----
+            // ---- in-block matches: rounds over the listed matches ----
             const uint32_t n_act = misc[3];
             for (;;) {
-                bool progress = false, left = false;
-                const uint32_t g = lane >> 3, sl = lane & 7;
-                const uint32_t gmask = 0xffu << (8 * g);
-                for (uint32_t base = warp * 4; base < n_act; base += (NT / 32) * 4) {
-                    const uint32_t i = base + g < n_act ? act_list[base + g] : n;
-                    const bool act = i < n && tstat[i] == 1;  // the same for the group's lanes
-                    uint32_t ml = 0, o = 0, so = 0, d = 1, we = 0;
-                    bool busy = false;
-                    if (act) {
-                        ml = tml[i];
-                        o = tpos[i] + tll[i];
-                        so = (uint32_t)(tsrc[i] - B);
-                        d = o - so;
-                        we = so + min(d, ml);  // periodic source window [so, we)
-                        for (uint32_t w = (so >> 5) + sl; w <= ((we - 1) >> 5); w += 8)
-                            busy |= (((volatile uint32_t*)pend)[w] & range_mask(w, so, we)) != 0;
-                    }
-                    const uint32_t bm = __ballot_sync(ACX_FULL, busy);  // every lane, active or not
-                    const bool ready = act && (bm & gmask) == 0;
-                    if (act && !ready) left = true;
-                    __threadfence_block();  // source reads after the readiness reads
-                    if (ready) {
-                        if (d >= ml) {
-                            copy_run8(sout, sout, so, o, ml, sl);
-                        } else {
-                            // out[o+k] = out[so + (k mod d)]: the source window only, so lanes are independent
-                            uint32_t r = sl % d;
-                            const uint32_t step = 8 % d;
-                            for (uint32_t k = sl; k < ml; k += 8) {
-                                sout[o + k] = sout[so + r];
-                                r += step;
-                                if (r >= d) r -= d;
-                            }
-                        }
-                    }
-                    __syncwarp();
-                    __threadfence_block();
-                    if (ready) {
-                        for (uint32_t w = (o >> 5) + sl; w <= ((o + ml - 1) >> 5); w += 8)
-                            atomicAnd(&pend[w], ~range_mask(w, o, o + ml));
-                        if (sl == 0) tstat[i] = 0;
-                        progress = true;
-                    }
-                }
-                const int any_left = grp_or<NT>(bid, left);
-                const int any_prog = grp_or<NT>(bid, progress);
+                const uint32_t r =
+                    NT > kLocThreads && n_act > kManyMatches
+                        ? match_pass<1>(tlit, n_act, 32 * warp, NT, sout, pend, tstat, tml, tpos, tll, tsrc, B, lane)
+                        : match_pass<8>(tlit, n_act, 4 * warp, NT / 8, sout, pend, tstat, tml, tpos, tll, tsrc, B, lane);
+                const int any_left = grp_or<NT>(bid, r & 1);
+                const int any_prog = grp_or<NT>(bid, r & 2);
                 if (!any_left || !any_prog) break;
             }
             // ---- whatever is still unresolved becomes pending pieces (for a
@@ -636,10 +721,10 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                     cnt += pieces_of(tml[i]);
                     nbytes += tml[i];
                 }
-            v3[0] = cnt; v3[1] = nbytes; v3[2] = 0;
-            block_scan3<NT>(v3, tot3, scanbuf, bid, tid);
-            npend = tot3[0];
-            pbytes = tot3[1];
+            v2[0] = cnt; v2[1] = nbytes;
+            block_scan<NT, 2>(v2, tot2, scanbuf, bid, tid);
+            npend = tot2[0];
+            pbytes = tot2[1];
             if (lvl) {
                 // the block's row of the level table (pieces of level <= l,
                 // a piece's level being its token's level byte clamped to
@@ -669,7 +754,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 }
             }
             {
-                uint32_t k = v3[0];
+                uint32_t k = v2[0];
                 for (uint32_t i = i0; i < i1; i++) {
                     if (!tstat[i]) continue;
                     const uint32_t o = tpos[i] + tll[i];
