@@ -70,11 +70,31 @@ __device__ __forceinline__ uint32_t rd32d(const uint8_t* p) {
     return (uint32_t)p[0] | ((uint32_t)p[1] << 8) | ((uint32_t)p[2] << 16) | ((uint32_t)p[3] << 24);
 }
 __device__ __forceinline__ uint64_t rd64d(const uint8_t* p) { return (uint64_t)rd32d(p) | ((uint64_t)rd32d(p + 4) << 32); }
+// N consecutive little-endian words at p, all loads before any use (words when
+// p is aligned, bytes otherwise).
+template <int N>
+__device__ __forceinline__ void rd_words(const uint8_t* p, uint32_t (&w)[N]) {
+    if (((uintptr_t)p & 3) == 0) {
+#pragma unroll
+        for (int i = 0; i < N; i++) w[i] = reinterpret_cast<const uint32_t*>(p)[i];
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; i++) w[i] = rd32d(p + 4 * i);
+    }
+}
 
 // Validate a format v1 archive held in device memory and build its decode
 // plan in the static scratch (one CTA).  The checks are the host plan
 // builder's: header, tables, index entries, payload descriptors.
-__global__ void __launch_bounds__(256) k_plan_small(const uint8_t* a, uint64_t len, uint8_t* base) {
+//
+// The kernel is bound by load round trips, so they are few and taken side by
+// side: a thread a block, its index entry and its four stream descriptors as
+// whole loads; the tables are summed and written by warps; offsets and maxima
+// over the blocks come from shared memory.  (With serial tables, byte loads and
+// one thread's walk over the blocks in global memory it took 135 us, half of a
+// 1 MB decode.)
+constexpr int kPlanThreads = 256;
+__global__ void __launch_bounds__(kPlanThreads) k_plan_small(const uint8_t* a, uint64_t len, uint8_t* base) {
     NaSummary* S = reinterpret_cast<NaSummary*>(base + kOffSummary);
     BlockDev* blk = reinterpret_cast<BlockDev*>(base + kOffPlan);
     uint32_t* tab = reinterpret_cast<uint32_t*>(base + kOffTab);
@@ -82,26 +102,33 @@ __global__ void __launch_bounds__(256) k_plan_small(const uint8_t* a, uint64_t l
     __shared__ int bad;            // 0 ok, -2 corrupt, -1 too large
     __shared__ uint64_t off_tab, off_idx, off_deps, total;
     __shared__ uint32_t nb, min_match, flags;
-    __shared__ uint16_t freq[4][256];
+    __shared__ uint16_t freq[4][256], cum[4][256];
     __shared__ uint32_t ok_tab[4];
-    const int tid = threadIdx.x;
+    __shared__ uint32_t b_bytes[kNaMaxBlocks], b_slots[kNaMaxBlocks];  // per block: stream bytes, piece slots
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
         bad = 0;
-        if (len < 64 || a[0] != 'A' || a[1] != 'C' || a[2] != 'X' || a[3] != '1' || rd16d(a + 4) != 1 ||
-            rd32d(a + 8) != kBlock) {
+        if (len < 64) {
             bad = -2;
         } else {
-            flags = rd16d(a + 6);
-            min_match = rd32d(a + 12);
-            total = rd64d(a + 16);
-            nb = rd32d(a + 24);
-            off_tab = rd64d(a + 32);
-            off_idx = rd64d(a + 40);
-            off_deps = rd64d(a + 48);
-            if (min_match < 4 || min_match > kBlock || (uint64_t)nb != (total + kBlock - 1) / kBlock) bad = -2;
-            else if (off_tab > len || len - off_tab < 2048) bad = -2;
-            else if (off_idx > len || (len - off_idx) / 40 < nb) bad = -2;
-            else if (nb > kNaMaxBlocks) bad = -1;
+            uint32_t h[14];
+            rd_words(a, h);
+            // "ACX1", version 1
+            if (h[0] != 0x31584341u || (h[1] & 0xffff) != 1 || h[2] != kBlock) {
+                bad = -2;
+            } else {
+                flags = h[1] >> 16;
+                min_match = h[3];
+                total = h[4] | (uint64_t)h[5] << 32;
+                nb = h[6];
+                off_tab = h[8] | (uint64_t)h[9] << 32;
+                off_idx = h[10] | (uint64_t)h[11] << 32;
+                off_deps = h[12] | (uint64_t)h[13] << 32;
+                if (min_match < 4 || min_match > kBlock || (uint64_t)nb != (total + kBlock - 1) / kBlock) bad = -2;
+                else if (off_tab > len || len - off_tab < 2048) bad = -2;
+                else if (off_idx > len || (len - off_idx) / 40 < nb) bad = -2;
+                else if (nb > kNaMaxBlocks) bad = -1;
+            }
         }
     }
     __syncthreads();
@@ -109,28 +136,55 @@ __global__ void __launch_bounds__(256) k_plan_small(const uint8_t* a, uint64_t l
         if (tid == 0) S->status = bad;
         return;
     }
-    for (uint32_t i = tid; i < 4 * 256; i += blockDim.x) freq[i >> 8][i & 255] = rd16d(a + off_tab + 2 * i);
+    for (uint32_t i = tid; i < 4 * 256; i += kPlanThreads) freq[i >> 8][i & 255] = rd16d(a + off_tab + 2 * i);
+    if (tid < (int)kNaMaxBlocks) b_bytes[tid] = b_slots[tid] = 0;
     __syncthreads();
-    if (tid < 4) {
-        uint32_t sum = 0;
-        for (int k = 0; k < 256; k++) sum += freq[tid][k];
-        ok_tab[tid] = sum == kM;
-        if (sum != 0 && sum != kM) bad = -2;
-    }
-    __syncthreads();
-    if (tid < 4 && ok_tab[tid]) {  // decode entries sym | (f-1) << 8 | (slot-c) << 20
-        uint32_t c = 0;
-        for (int k = 0; k < 256; k++) {
-            const uint32_t f = freq[tid][k];
-            for (uint32_t r = 0; r < f; r++) tab[tid * kM + c + r] = (uint32_t)k | ((f - 1) << 8) | (r << 20);
-            c += f;
+    if (warp < 4) {  // table `warp`: its sum and each symbol's first slot
+        uint32_t own = 0;
+        for (int k = 0; k < 8; k++) own += freq[warp][8 * lane + k];
+        uint32_t inc = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(ACX_FULL, inc, o);
+            if (lane >= o) inc += y;
+        }
+        const uint32_t sum = __shfl_sync(ACX_FULL, inc, 31);
+        uint32_t c = inc - own;
+        for (int k = 0; k < 8; k++) {
+            cum[warp][8 * lane + k] = (uint16_t)c;  // (used only when the sum is kM)
+            c += freq[warp][8 * lane + k];
+        }
+        if (lane == 0) {
+            ok_tab[warp] = sum == kM;
+            if (sum != 0 && sum != kM) bad = -2;
         }
     }
-    for (uint32_t b = tid; b < nb; b += blockDim.x) {
-        const uint8_t* e = a + off_idx + 40 * (uint64_t)b;
-        const uint64_t poff = rd64d(e);
-        const uint32_t plen = rd32d(e + 8), n_tok = rd32d(e + 12), raw = rd32d(e + 16);
-        const uint32_t dep_off = rd32d(e + 20), n_deps = rd32d(e + 24);
+    __syncthreads();
+    // decode entries sym | (f-1) << 8 | (slot-c) << 20: a slot's symbol is the
+    // last one that starts at or before it (symbols that do not occur start
+    // where the next one does)
+    for (uint32_t i = tid; i < 4 * kM; i += 4 * kPlanThreads) {
+        uint32_t k[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (uint32_t h = 128; h; h >>= 1)
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const uint32_t j = i + u * kPlanThreads;
+                if (cum[j / kM][k[u] + h] <= j % kM) k[u] += h;
+            }
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const uint32_t j = i + u * kPlanThreads, t = j / kM;
+            if (ok_tab[t]) tab[j] = k[u] | (uint32_t)(freq[t][k[u]] - 1) << 8 | (j % kM - cum[t][k[u]]) << 20;
+        }
+    }
+    const uint32_t b = tid;
+    BlockDev bd{};
+    if (b < nb) {
+        uint32_t e[7];
+        rd_words(a + off_idx + 40 * (uint64_t)b, e);
+        const uint64_t poff = e[0] | (uint64_t)e[1] << 32;
+        const uint32_t plen = e[2], n_tok = e[3], raw = e[4], dep_off = e[5], n_deps = e[6];
         const uint64_t B = (uint64_t)b * kBlock;
         const uint64_t R = total - B < kBlock ? total - B : kBlock;
         bool ok = raw == R && !(off_deps == 0 && (dep_off || n_deps));
@@ -147,9 +201,10 @@ __global__ void __launch_bounds__(256) k_plan_small(const uint8_t* a, uint64_t l
             }
         }
         ok = ok && !(poff & 15) && !(plen & 15) && plen >= 48 && poff <= len && len - poff >= plen;
-        BlockDev bd{};
+        uint64_t soff = 0;
         if (ok) {
-            const uint8_t* pay = a + poff;
+            uint32_t d[12];
+            rd_words(a + poff, d);
             bd.payload = poff;
             bd.raw_len = raw;
             bd.n_tok = n_tok;
@@ -157,12 +212,12 @@ __global__ void __launch_bounds__(256) k_plan_small(const uint8_t* a, uint64_t l
                 bd.dep_off = dslot;
                 bd.n_deps = n_deps;
             }
-            uint64_t off = 48, soff = 0;
-            for (int s = 0; s < 4 && ok; s++) {
-                const uint8_t* d = pay + 12 * s;
-                const uint32_t sraw = rd32d(d), enc = rd32d(d + 4);
-                const uint8_t mode = d[8], K = d[9];
-                if (rd16d(d + 10) != 0 || sraw > kMaxStreamRaw || off + enc > plen) { ok = false; break; }
+            uint64_t off = 48;
+#pragma unroll
+            for (int s = 0; s < 4; s++) {
+                const uint32_t sraw = d[3 * s], enc = d[3 * s + 1];
+                const uint8_t mode = (uint8_t)d[3 * s + 2], K = (uint8_t)(d[3 * s + 2] >> 8);
+                if (d[3 * s + 2] >> 16 || sraw > kMaxStreamRaw || off + enc > plen) ok = false;
                 if (mode == 0) {
                     if (enc != sraw || K != 0) ok = false;
                 } else if (mode == 1) {
@@ -191,38 +246,53 @@ __global__ void __launch_bounds__(256) k_plan_small(const uint8_t* a, uint64_t l
             // (the regular decode finds such a block corrupt too)
             ok = ok && n_tok <= raw / min_match + 1;
             bd.n_new = bd.s_raw[kOff] / 5;
-            bd.scratch = soff;  // this block's stream bytes; offsets are assigned below
         }
-        if (!ok) bad = -2;
-        blk[b] = bd;
+        if (ok) {
+            b_bytes[b] = (uint32_t)soff;  // (four streams of at most kMaxStreamRaw bytes)
+            b_slots[b] = n_tok + kSpanSlack;
+        } else {
+            bad = -2;
+        }
     }
     __syncthreads();
-    if (tid == 0) {
-        int st = bad;
-        uint64_t scratch = 0, slots = 0;
-        uint32_t max_tok = 1, max_lenb = 1, max_lit = 0;
-        for (uint32_t b = 0; b < nb && !st; b++) {
-            BlockDev& bd = blk[b];
-            const uint64_t sz = bd.scratch;
-            bd.scratch = scratch;
-            bd.span_base = (uint32_t)slots;
-            scratch += sz;
-            slots += bd.n_tok + kSpanSlack;
-            max_tok = max(max_tok, bd.n_tok);
-            max_lenb = max(max_lenb, bd.s_raw[kLen]);
-            max_lit = max(max_lit, bd.s_raw[kLit]);
+    if (bad) {
+        if (tid == 0) S->status = bad;
+        return;
+    }
+    if (b < nb) {
+        uint32_t scratch = 0, slots = 0;  // (64 blocks: both fit 32 bits)
+        for (uint32_t k = 0; k < b; k++) {
+            scratch += b_bytes[k];
+            slots += b_slots[k];
         }
-        if (!st && (scratch + 64 > kNaStreamBytes || slots > kNaSpanSlots)) st = -1;
-        S->status = st;
-        S->n_blocks = nb;
-        S->min_match = min_match;
-        S->max_tok = max_tok;
-        S->max_lenb = max_lenb;
-        S->max_lit = max_lit;
-        S->total = total;
-        S->has_deps = off_deps != 0;
-        S->span_slots = slots;
-        S->stream_bytes = scratch;
+        bd.scratch = scratch;
+        bd.span_base = slots;
+        blk[b] = bd;
+    }
+    if (warp < 2) {  // the summary: block b is lane b & 31 of warp b >> 5
+        __shared__ uint32_t part[2][5];
+        const uint32_t v[5] = {b < nb ? b_bytes[b] : 0, b < nb ? b_slots[b] : 0, bd.n_tok, bd.s_raw[kLen], bd.s_raw[kLit]};
+        uint32_t r[5];
+        r[0] = __reduce_add_sync(ACX_FULL, v[0]);
+        r[1] = __reduce_add_sync(ACX_FULL, v[1]);
+#pragma unroll
+        for (int k = 2; k < 5; k++) r[k] = __reduce_max_sync(ACX_FULL, v[k]);
+        if (lane == 0)
+            for (int k = 0; k < 5; k++) part[warp][k] = r[k];
+        asm volatile("bar.sync 1, 64;" ::: "memory");  // (warps 0 and 1)
+        if (tid == 0) {
+            const uint64_t scratch = (uint64_t)part[0][0] + part[1][0], slots = (uint64_t)part[0][1] + part[1][1];
+            S->status = scratch + 64 > kNaStreamBytes || slots > kNaSpanSlots ? -1 : 0;
+            S->n_blocks = nb;
+            S->min_match = min_match;
+            S->max_tok = max(1u, max(part[0][2], part[1][2]));
+            S->max_lenb = max(1u, max(part[0][3], part[1][3]));
+            S->max_lit = max(part[0][4], part[1][4]);
+            S->total = total;
+            S->has_deps = off_deps != 0;
+            S->span_slots = slots;
+            S->stream_bytes = scratch;
+        }
     }
 }
 
@@ -253,7 +323,7 @@ extern "C" int aceapex_decode_noalloc(const void* d_arc, uint64_t arc_len, void*
         base = g_na_base[dev];
     }
     cudaStream_t st = (cudaStream_t)stream;
-    k_plan_small<<<1, 256, 0, st>>>((const uint8_t*)d_arc, arc_len, base);
+    k_plan_small<<<1, kPlanThreads, 0, st>>>((const uint8_t*)d_arc, arc_len, base);
     if (cudaGetLastError() != cudaSuccess) return ACEAPEX_E_CUDA;
     NaSummary S;
     if (cudaMemcpyAsync(&S, base + kOffSummary, sizeof S, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
