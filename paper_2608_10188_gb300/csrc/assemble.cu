@@ -521,6 +521,8 @@ __global__ void __launch_bounds__(kExtThreads) k_external(JobDev job) {
         job.counters[kTrace + 1] = (uint32_t)t;
         job.counters[kTrace + 2] = (uint32_t)(t >> 32);
     }
+    const uint64_t pieces = *((volatile const uint32_t*)&job.counters[kStatPending]);
+    if (pieces == 0) return;  // (every CTA reads the same final count)
     // round 0: pieces handed out in order; a lane waits for the sources that
     // lower pieces are about to finish, without limit unless wait_ns sets one:
     // then it defers its piece to the rounds below.  The order is the output
@@ -572,7 +574,6 @@ __global__ void __launch_bounds__(kExtThreads) k_external(JobDev job) {
                 n_lv = 0;
             }
         }
-        const uint64_t pieces = *((volatile const uint32_t*)&job.counters[kStatPending]);
         const uint64_t per_part = (uint64_t)job.n_items * kPartPieces;
         const uint32_t parts = (uint32_t)max((pieces + per_part - 1) / per_part, (uint64_t)1);
         const uint64_t n_tickets = (uint64_t)job.n_items * parts;
@@ -761,7 +762,8 @@ cudaError_t launch_external(const JobDev& job, int grid, cudaStream_t st) {
     return coop_ordered(st, [](void* p) -> cudaError_t {
         const Arg* a = static_cast<const Arg*>(p);
         cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(a->grid);
+        // two CTAs a block take all of its parts at once
+        cfg.gridDim = dim3((uint32_t)std::min<uint64_t>((uint64_t)a->grid, 2ull * a->job->n_items));
         cfg.blockDim = dim3(kExtThreads);
         cfg.dynamicSmemBytes = 0;
         cfg.stream = a->st;
