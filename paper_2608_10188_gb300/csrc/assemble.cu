@@ -41,6 +41,7 @@ namespace acx {
 template <int NT>
 __global__ void __launch_bounds__(NT, NT == kLocThreads ? 6 : NT == kLocWide ? 3 : 1) k_local(JobDev job) {
     extern __shared__ __align__(128) uint8_t sm[];
+    grid_dependency_wait();  // the entropy stage's streams
     local_worker<NT>(job, sm, 0, threadIdx.x);
 }
 
@@ -701,8 +702,7 @@ template <int NT>
 static cudaError_t launch_local_nt(const JobDev& job, int grid, size_t smem, cudaStream_t st) {
     const cudaError_t e = local_attrs<NT>(smem);
     if (e != cudaSuccess) return e;
-    k_local<NT><<<grid, NT, smem, st>>>(job);
-    return cudaGetLastError();
+    return launch_dependent(k_local<NT>, grid, NT, smem, st, job);
 }
 
 cudaError_t launch_local(const JobDev& job, int grid, cudaStream_t st) {

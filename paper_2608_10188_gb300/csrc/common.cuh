@@ -127,6 +127,12 @@ __device__ __forceinline__ void tma_load_1d(void* dst, const void* src, uint32_t
         : "memory");
 }
 
+// Programmatic dependent launch: the kernel launched behind this one may take
+// its places on the SMs from here on; it waits (grid_dependency_wait) until
+// this grid has completed and its writes are visible before it reads them.
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ int find_arc(const JobDev& job, uint32_t item) {
     if (!job.arcs) return 0;
     int lo = 0, hi = (int)job.n_arcs - 1;

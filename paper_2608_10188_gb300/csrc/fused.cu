@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kFusedMaxThreads, 1) k_fused(JobDev job, int G
             const uint32_t tk = __shfl_sync(ACX_FULL, t0, 0);
             if (tk >= n_a) break;
             const uint32_t item = J.order ? J.order[tk] : tk;
-            rans_block(job, 0, J, item_ref(J, item), kRansAll, tab0_s, ring_s, smem_u32(sm + F.stage) + warp * kStageBytes,
+            rans_block(job, 0, J, item_ref(J, item), kRansAll, TabLoad{nullptr, 0}, tab0_s, ring_s, smem_u32(sm + F.stage) + warp * kStageBytes,
                        &bars[0], &bars[kSlots], seq, sphase, lane, deadline);
             // publish: every lane's stream stores, then the flag (a corrupt
             // block is published too; its local pass finds it corrupt)

@@ -8,6 +8,25 @@
 
 namespace acx {
 
+// Launch a kernel that begins with grid_dependency_wait() and may come up while
+// the kernel before it on the stream still runs (programmatic dependent launch):
+// its launch, and what it does before the wait, hide behind that kernel (10 KB
+// file 75 -> 70 us, 1 MB without allocations 154 -> 145, 64 MiB genome 231 -> 224).
+template <class K, class... A>
+cudaError_t launch_dependent(K kernel, int grid, int block, size_t smem, cudaStream_t st, const A&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Clears counters[0, n_counters) and the statistics/list/barrier words, and
 // errs[0, n_errs) (status words that the kernels set).
 cudaError_t launch_prologue(uint32_t* counters, uint32_t n_counters, cudaStream_t st, int* errs = nullptr,

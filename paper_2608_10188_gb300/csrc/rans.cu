@@ -10,6 +10,7 @@ namespace acx {
 
 // Start of a decode call: every ticket and statistic restarts at zero.
 __global__ void k_prologue(uint32_t* counters, uint32_t n_counters, int* errs, uint32_t n_errs) {
+    grid_launch_dependents();
     for (uint32_t i = threadIdx.x; i < n_counters; i += blockDim.x) counters[i] = 0;
     for (uint32_t i = threadIdx.x; i < n_errs; i += blockDim.x) errs[i] = 0;
     if (threadIdx.x < kLvStripes) counters[kLvTickets + threadIdx.x] = 0;
@@ -34,6 +35,8 @@ __global__ void __launch_bounds__(kRansWarps * 32) k_rans(JobDev job) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (lane < kSlots) mbar_init(&S.bar[warp][lane], 1);
     if (lane == kSlots) mbar_init(&S.sbar[warp], 1);
+    if (threadIdx.x < 4) mbar_init(&S.tbar[threadIdx.x], 1);
+    grid_launch_dependents();
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if (threadIdx.x == 0) {
         const uint64_t target = (uint64_t)blockIdx.x * job.n_items / gridDim.x;
@@ -41,8 +44,8 @@ __global__ void __launch_bounds__(kRansWarps * 32) k_rans(JobDev job) {
         S.arc = -1;
     }
     __syncthreads();
-    const uint64_t deadline = gtimer() + kCopyWaitNs;  // the entropy stage waits only for its copies
-    uint32_t seq = 0, sphase = 0;
+    uint64_t deadline = 0;  // the entropy stage waits only for its copies
+    uint32_t seq = 0, sphase = 0, tphase = 1;
     uint32_t* tickets = job.counters + 3;
     const uint32_t ring_s = ring_addr(S, warp);
     for (;;) {
@@ -50,11 +53,24 @@ __global__ void __launch_bounds__(kRansWarps * 32) k_rans(JobDev job) {
         if (a < 0) break;
         const ArcJob J = load_arc(job, a);
         if (S.arc != a) {
-            const uint4* src = reinterpret_cast<const uint4*>(J.dtab);
-            uint4* dst = reinterpret_cast<uint4*>(&S.tab[0][0]);
-            for (int i = threadIdx.x; i < (int)(4 * kM / 4); i += blockDim.x) dst[i] = src[i];
+            // (every warp has left the tables of the archive before)
+            if (threadIdx.x == 0) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                for (int k = 0; k < 4; k++) {
+                    const int s = k == 0 ? kLit : k - 1;  // the literals' first: the longest streams
+                    mbar_arrive_tx(&S.tbar[s], 4 * kM);
+                    tma_load_1d(S.tab[s], J.dtab + s * kM, 4 * kM, &S.tbar[s]);
+                }
+            }
+            tphase ^= 1;
             __syncthreads();
             if (threadIdx.x == 0) S.arc = a;
+        }
+        const TabLoad T{S.tbar, tphase};
+        if (!deadline) {
+            // (plans and tables do not depend on the kernel before, tickets do)
+            grid_dependency_wait();
+            deadline = gtimer() + kCopyWaitNs;
         }
         // tickets: the blocks, or (rans_parts) their literals, then their other
         // parts; a lone archive's first run of every warp is its own, so that
@@ -76,9 +92,13 @@ __global__ void __launch_bounds__(kRansWarps * 32) k_rans(JobDev job) {
             if (tk >= n_a) break;
             const uint32_t turn = tk / n_blk, i = tk - turn * n_blk;
             const uint32_t part = job.rans_parts == 1 ? kRansAll : kRansParts - 1 - turn;
-            rans_block(job, a, J, item_ref(J, J.order ? J.order[i] : i), part, smem_u32(&S.tab[0][0]), ring_s,
+            rans_block(job, a, J, item_ref(J, J.order ? J.order[i] : i), part, T, smem_u32(&S.tab[0][0]), ring_s,
                        smem_u32(&S.stage[warp][0]), &S.bar[warp][0], &S.sbar[warp], seq, sphase, lane, deadline);
         }
+        // a warp without work has not waited for the tables: their copies land
+        // before the CTA leaves or the next archive's go out
+        if (warp == 0)
+            for (int s = 0; s < 4; s++) wait_table(T, s, deadline);
         if (job.n_arcs == 1) break;
         __syncthreads();
         if (warp == 0) {
@@ -133,8 +153,7 @@ cudaError_t launch_rans(const JobDev& job_in, int grid, cudaStream_t st) {
     const uint64_t per_cta = (uint64_t)kRansWarps * (job.chunk ? job.chunk : 1);
     const uint64_t need = ((uint64_t)job.n_items * job.rans_parts + per_cta - 1) / per_cta;
     if (need <= (uint64_t)noted_sm_count()) grid = std::min(grid, noted_sm_count());
-    k_rans<<<grid, kRansWarps * 32, sm, st>>>(job);
-    return cudaGetLastError();
+    return launch_dependent(k_rans, grid, kRansWarps * 32, sm, st, job);
 }
 
 int rans_occupancy() {

@@ -37,6 +37,7 @@ struct RansSmem {
     uint64_t bar[kRansWarps][kSlots];
     alignas(16) uint8_t stage[kRansWarps][kStageBytes];
     uint64_t sbar[kRansWarps];                         // short-stream staging barrier of each warp
+    uint64_t tbar[4];                                  // the four tables' copies
     int arc;                                           // archive whose tables are loaded
     int next_arc;
 };
@@ -45,6 +46,24 @@ struct RansSmem {
 // byte offset is OR-ed onto it.
 __device__ __forceinline__ uint32_t ring_addr(RansSmem& S, int w) {
     return ((smem_u32(S.ringspace) + kRingMask) & ~(uint32_t)kRingMask) + (uint32_t)w * (2 * kRingWords);
+}
+
+// Decode tables on their way into shared memory: a barrier per stream type
+// (nullptr: they are there), and the phase of this load.  A warp waits for a
+// table when its first words and states are on their way too; loaded by all
+// threads before any work, the 64 KiB cost every CTA of a batch 55 us over its
+// archives (96 files: 753 -> 698 us).
+struct TabLoad {
+    uint64_t* bar;
+    uint32_t phase;
+};
+__device__ __forceinline__ bool wait_table(const TabLoad& T, int s, uint64_t deadline) {
+    if (!T.bar) return true;
+    uint32_t spins = 0;
+    bool ok = true;
+    while (!mbar_try_wait(&T.bar[s], T.phase))
+        if ((++spins & 1023) == 0 && gtimer() > deadline) { ok = false; break; }
+    return __all_sync(ACX_FULL, ok);
 }
 
 __device__ __forceinline__ bool wait_chunk(uint64_t* bar, uint32_t q, uint64_t deadline) {
@@ -95,7 +114,7 @@ __device__ __forceinline__ void rans_renorm(uint32_t& x, uint32_t& rb, uint32_t 
 // mbarrier phase bookkeeping across streams).  Returns false on a format
 // violation (word overrun, end states != 2^16) or an expired wait.
 template <int S>
-__device__ __forceinline__ bool rans_stream(uint32_t tab_s, const uint8_t* __restrict__ body, uint32_t enc,
+__device__ __forceinline__ bool rans_stream(const TabLoad& T, int type, uint32_t tab_s, const uint8_t* __restrict__ body, uint32_t enc,
                                             uint32_t n, uint32_t K, uint8_t* __restrict__ out, uint32_t ring_s,
                                             uint32_t stage_s, uint64_t* bar, uint32_t& seq, int lane,
                                             uint64_t deadline) {
@@ -121,6 +140,7 @@ __device__ __forceinline__ bool rans_stream(uint32_t tab_s, const uint8_t* __res
     uint32_t issued = 0, ready = 0;
     for (; issued < nchunks && issued < (uint32_t)kSlots; issued++)
         issue_chunk(ring_s, bar, words, seq0 + issued, issued, wbytes, lane);
+    ok = wait_table(T, type, deadline) && ok;
     const uint32_t lt_mask = (1u << lane) - 1;
     uint32_t p = 0;
     const uint32_t steps = ok ? (n + K - 1) / K : 0;
@@ -213,15 +233,15 @@ __device__ __forceinline__ bool rans_stream(uint32_t tab_s, const uint8_t* __res
 // The wide-lane variants are rare (archives encoded with more than 32
 // lanes): out of line, so that they do not raise the kernel's register
 // pressure.
-static __device__ __noinline__ bool rans_stream2(uint32_t tab_s, const uint8_t* body, uint32_t enc, uint32_t n, uint32_t K,
+static __device__ __noinline__ bool rans_stream2(const TabLoad& T, int type, uint32_t tab_s, const uint8_t* body, uint32_t enc, uint32_t n, uint32_t K,
                                           uint8_t* out, uint32_t ring_s, uint32_t stage_s, uint64_t* bar,
                                           uint32_t& seq, int lane, uint64_t deadline) {
-    return rans_stream<2>(tab_s, body, enc, n, K, out, ring_s, stage_s, bar, seq, lane, deadline);
+    return rans_stream<2>(T, type, tab_s, body, enc, n, K, out, ring_s, stage_s, bar, seq, lane, deadline);
 }
-static __device__ __noinline__ bool rans_stream4(uint32_t tab_s, const uint8_t* body, uint32_t enc, uint32_t n, uint32_t K,
+static __device__ __noinline__ bool rans_stream4(const TabLoad& T, int type, uint32_t tab_s, const uint8_t* body, uint32_t enc, uint32_t n, uint32_t K,
                                           uint8_t* out, uint32_t ring_s, uint32_t stage_s, uint64_t* bar,
                                           uint32_t& seq, int lane, uint64_t deadline) {
-    return rans_stream<4>(tab_s, body, enc, n, K, out, ring_s, stage_s, bar, seq, lane, deadline);
+    return rans_stream<4>(T, type, tab_s, body, enc, n, K, out, ring_s, stage_s, bar, seq, lane, deadline);
 }
 
 // Which of a block's short streams (cmd, len, off) decode side by side on one
@@ -249,7 +269,7 @@ __device__ __forceinline__ uint32_t short_group(const BlockDev& bd) {
 // warp: stream g runs on lanes [lo_g, lo_g + K_g) with its own word pointer;
 // their words are staged whole into the warp's ring by TMA.  Returns false on
 // a format violation or an expired wait.
-__device__ __forceinline__ bool rans_short(uint32_t mask, uint32_t tab0_s, const BlockDev& bd, const uint8_t* pay,
+__device__ __forceinline__ bool rans_short(const TabLoad& T, uint32_t mask, uint32_t tab0_s, const BlockDev& bd, const uint8_t* pay,
                                            uint8_t* scr, uint32_t ring_s, uint64_t* sbar, uint32_t& sphase, int lane,
                                            uint64_t deadline) {
     uint32_t lo[3], K[3], W[3], hdr[3], roff[3], nw_bytes[3];
@@ -304,6 +324,8 @@ __device__ __forceinline__ bool rans_short(uint32_t mask, uint32_t tab0_s, const
         sphase++;
         if (!__all_sync(ACX_FULL, w)) return false;
     }
+    for (int g = 0; g < 3; g++)
+        if ((mask & (1u << g)) && !wait_table(T, g, deadline)) return false;
     ok = __all_sync(ACX_FULL, ok);
     const uint32_t lt_mask = (1u << lane) - 1;
     uint32_t p = 0;
@@ -352,12 +374,13 @@ constexpr uint32_t kRansParts = 3, kRansAll = 3;
 // Entropy-decode one work item's streams, or one part of them (one warp), into
 // its decoded-stream scratch: the short streams that fit the warp together
 // side by side, then the rest one by one (the literal stream is skipped by a
-// parse-only job).  tab0_s is the shared address of the four decode tables;
+// parse-only job).  tab0_s is the shared address of the four decode tables, T
+// their loads;
 // bar (kSlots barriers), sbar, the ring and the symbol stage (kStageBytes,
 // 16-aligned) are the warp's own.  A corrupt stream sets the job's (and the
 // archive's) error status.
 __device__ __forceinline__ void rans_block(const JobDev& job, int a, const ArcJob& J, const ItemRef& ir,
-                                           uint32_t part, uint32_t tab0_s, uint32_t ring_s, uint32_t stage_s,
+                                           uint32_t part, const TabLoad& T, uint32_t tab0_s, uint32_t ring_s, uint32_t stage_s,
                                            uint64_t* bar, uint64_t* sbar, uint32_t& seq, uint32_t& sphase, int lane,
                                            uint64_t deadline) {
     const uint32_t b = ir.blk;
@@ -374,7 +397,7 @@ __device__ __forceinline__ void rans_block(const JobDev& job, int a, const ArcJo
     bool ok = true;
     int fs = 0;
     if (together && part != 1 && part != 2) {
-        ok = rans_short(together, tab0_s, bd, pay, scr, ring_s, sbar, sphase, lane, deadline);
+        ok = rans_short(T, together, tab0_s, bd, pay, scr, ring_s, sbar, sphase, lane, deadline);
         mask &= ~together;
     }
     for (int s = 0; s < 4 && ok; s++) {
@@ -387,9 +410,9 @@ __device__ __forceinline__ void rans_block(const JobDev& job, int a, const ArcJo
         if (bd.rans_mask & (1u << s)) {
             const uint32_t K = bd.s_K[s];
             const uint32_t tb = tab0_s + s * kM * 4;
-            if (K <= 32) ok = rans_stream<1>(tb, body, bd.s_enc[s], n, K, o, ring_s, stage_s, bar, seq, lane, deadline);
-            else if (K == 64) ok = rans_stream2(tb, body, bd.s_enc[s], n, K, o, ring_s, stage_s, bar, seq, lane, deadline);
-            else ok = rans_stream4(tb, body, bd.s_enc[s], n, K, o, ring_s, stage_s, bar, seq, lane, deadline);
+            if (K <= 32) ok = rans_stream<1>(T, s, tb, body, bd.s_enc[s], n, K, o, ring_s, stage_s, bar, seq, lane, deadline);
+            else if (K == 64) ok = rans_stream2(T, s, tb, body, bd.s_enc[s], n, K, o, ring_s, stage_s, bar, seq, lane, deadline);
+            else ok = rans_stream4(T, s, tb, body, bd.s_enc[s], n, K, o, ring_s, stage_s, bar, seq, lane, deadline);
         } else {
             copy_stored(body, o, n, lane);
         }
