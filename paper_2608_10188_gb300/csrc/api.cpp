@@ -5,6 +5,8 @@
 #include <string.h>
 
 #include <algorithm>
+#include <memory>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -45,6 +47,7 @@ int aceapex_ctx_create(int device, const aceapex_dec_params* params, aceapex_ctx
     if (cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
         cudaMalloc(&c->counters, kMaxCounters * sizeof(uint32_t)) != cudaSuccess ||
         cudaMalloc(&c->d_err, 4 * sizeof(int)) != cudaSuccess ||
+        cudaMallocHost(&c->h_err, kStatusWords * sizeof(int)) != cudaSuccess ||
         cudaMemset(c->counters, 0, kMaxCounters * sizeof(uint32_t)) != cudaSuccess ||
         cudaMemset(c->d_err, 0, 4 * sizeof(int)) != cudaSuccess) {
         aceapex_ctx_destroy(c);
@@ -84,6 +87,7 @@ int aceapex_ctx_destroy(aceapex_ctx* c) {
     c->lvl_list.release();
     if (c->counters) cudaFree(c->counters);
     if (c->d_err) cudaFree(c->d_err);
+    if (c->h_err) cudaFreeHost(c->h_err);
     for (auto& ev : c->pipe_ev) cudaEventDestroy(ev);
     if (c->s_up) cudaStreamDestroy(c->s_up);
     if (c->s_down) cudaStreamDestroy(c->s_down);
@@ -124,59 +128,61 @@ int aceapex_encode_ex(const uint8_t* src, uint64_t n, const aceapex_enc_params* 
 
 void aceapex_free(void* p) { free(p); }
 
-int aceapex_archive_open(aceapex_ctx* c, const void* d_arc, const void* h_arc, uint64_t len, aceapex_archive** out) {
+int aceapex_archive_open(aceapex_ctx* c, const void* d_arc, const void* h_arc, uint64_t len, aceapex_archive** out) try {
     if (!c || !out || !h_arc || !d_arc) return fail(c, ACEAPEX_E_ARG, "archive_open: null argument");
     *out = nullptr;
     cudaSetDevice(c->device);
-    aceapex_archive* A = new (std::nothrow) aceapex_archive();
-    if (!A) return fail(c, ACEAPEX_E_NOMEM, "archive_open: host allocation");
+    std::unique_ptr<aceapex_archive, int (*)(aceapex_archive*)> guard(new aceapex_archive(), aceapex_archive_close);
+    aceapex_archive* A = guard.get();
     std::string why;
     if (build_plan((const uint8_t*)h_arc, len, &A->plan, &why) != 0) {
-        delete A;
         return fail(c, ACEAPEX_E_CORRUPT, "archive_open: " + why);
     }
     A->ctx = c;
     A->d_arc = d_arc;
-    const size_t nb = A->plan.blk.size();
-    cudaError_t e = cudaMalloc(&A->d_blk, std::max<size_t>(nb, 1) * sizeof(BlockDev));
-    if (e == cudaSuccess) e = cudaMalloc(&A->d_dtab, 4 * kM * sizeof(uint32_t));
-    if (e == cudaSuccess && nb) e = cudaMemcpy(A->d_blk, A->plan.blk.data(), nb * sizeof(BlockDev), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(A->d_dtab, A->plan.dtab.data(), 4 * kM * sizeof(uint32_t), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && A->plan.has_deps) {
-        const size_t nd = std::max<size_t>(A->plan.deps.size(), 1);
-        e = cudaMalloc(&A->d_deps, nd * sizeof(uint32_t));
-        if (e == cudaSuccess && !A->plan.deps.empty())
-            e = cudaMemcpy(A->d_deps, A->plan.deps.data(), A->plan.deps.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
-    }
-    if (e == cudaSuccess && nb) {
+    // the archive's device tables in one allocation, filled by one copy: an
+    // archive that is opened for one decode pays for each driver call
+    const size_t nb = A->plan.blk.size(), nd = A->plan.has_deps ? std::max<size_t>(A->plan.deps.size(), 1) : 0;
+    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t o_blk = up(4 * kM * sizeof(uint32_t)), o_order = o_blk + up(nb * sizeof(BlockDev));
+    const size_t o_deps = o_order + up(nb * sizeof(uint32_t)), bytes = o_deps + nd * sizeof(uint32_t);
+    std::vector<uint8_t> h(bytes, 0);
+    memcpy(h.data(), A->plan.dtab.data(), 4 * kM * sizeof(uint32_t));
+    if (nb) {
+        memcpy(h.data() + o_blk, A->plan.blk.data(), nb * sizeof(BlockDev));
         // entropy-stage hand-out order: most symbols first (longest-first
         // scheduling keeps the last wave of the persistent warps short)
-        std::vector<uint32_t> ord(nb);
+        uint32_t* ord = reinterpret_cast<uint32_t*>(h.data() + o_order);
         std::vector<uint64_t> key(nb);
         for (size_t b = 0; b < nb; b++) {
             const BlockDev& bd = A->plan.blk[b];
             ord[b] = (uint32_t)b;
             key[b] = (uint64_t)bd.s_raw[0] + bd.s_raw[1] + bd.s_raw[2] + bd.s_raw[3];
         }
-        std::stable_sort(ord.begin(), ord.end(), [&](uint32_t x, uint32_t y) { return key[x] > key[y]; });
-        e = cudaMalloc(&A->d_order, nb * sizeof(uint32_t));
-        if (e == cudaSuccess) e = cudaMemcpy(A->d_order, ord.data(), nb * sizeof(uint32_t), cudaMemcpyHostToDevice);
+        std::stable_sort(ord, ord + nb, [&](uint32_t x, uint32_t y) { return key[x] > key[y]; });
     }
-    if (e != cudaSuccess) {
-        aceapex_archive_close(A);
-        return cuda_fail(c, e, "archive_open");
+    if (A->plan.has_deps && !A->plan.deps.empty())
+        memcpy(h.data() + o_deps, A->plan.deps.data(), A->plan.deps.size() * sizeof(uint32_t));
+    cudaError_t e = cudaMalloc(&A->d_tables, bytes);
+    if (e == cudaSuccess) {
+        uint8_t* base = (uint8_t*)A->d_tables;
+        A->d_dtab = (uint32_t*)base;
+        A->d_blk = (BlockDev*)(base + o_blk);
+        if (nb) A->d_order = (uint32_t*)(base + o_order);
+        if (A->plan.has_deps) A->d_deps = (uint32_t*)(base + o_deps);
+        e = cudaMemcpy(base, h.data(), bytes, cudaMemcpyHostToDevice);
     }
-    *out = A;
+    if (e != cudaSuccess) return cuda_fail(c, e, "archive_open");
+    *out = guard.release();
     return ACEAPEX_OK;
+} catch (const std::bad_alloc&) {
+    return fail(c, ACEAPEX_E_NOMEM, "archive_open: host allocation");
 }
 
 int aceapex_archive_close(aceapex_archive* A) {
     if (!A) return ACEAPEX_E_ARG;
     if (A->ctx) cudaSetDevice(A->ctx->device);
-    if (A->d_blk) cudaFree(A->d_blk);
-    if (A->d_dtab) cudaFree(A->d_dtab);
-    if (A->d_deps) cudaFree(A->d_deps);
-    if (A->d_order) cudaFree(A->d_order);
+    if (A->d_tables) cudaFree(A->d_tables);
     if (A->d_slot) cudaFree(A->d_slot);
     delete A->midx;
     delete A;
@@ -392,11 +398,11 @@ std::string acx::device_error_text(const int h[3]) {
 }
 
 int acx::ctx_read_status(aceapex_ctx* c, cudaStream_t st) {
-    cudaError_t e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(c, e, "stream synchronize");
-    int h[4] = {0, 0, 0, 0};
-    if ((e = cudaMemcpy(h, c->d_err, sizeof(h), cudaMemcpyDeviceToHost)) != cudaSuccess)
-        return cuda_fail(c, e, "error word");
+    // the status words come back behind the work, so one wait covers both
+    cudaError_t e = cudaMemcpyAsync(c->h_err, c->d_err, 4 * sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e != cudaSuccess) return cuda_fail(c, e, "error word");
+    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(c, e, "stream synchronize");
+    const int h[4] = {c->h_err[0], c->h_err[1], c->h_err[2], c->h_err[3]};
     if (h[0]) {
         cudaMemset(c->d_err, 0, sizeof(h));
         return fail(c, h[0], device_error_text(h));

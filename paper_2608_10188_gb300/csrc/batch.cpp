@@ -230,11 +230,12 @@ int aceapex_batch_wait(aceapex_batch* B, void* stream, aceapex_batch_item* items
     if (!B) return ACEAPEX_E_ARG;
     aceapex_ctx* c = B->ctx;
     cudaSetDevice(c->device);
-    cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "stream synchronize");
-    if ((e = cudaMemcpy(B->h_errs.data(), B->d_errs, B->h_errs.size() * sizeof(int), cudaMemcpyDeviceToHost)) !=
-        cudaSuccess)
-        return cuda_fail(c, e, "status words");
+    // the status words come back behind the work, so one wait covers both
+    cudaError_t e = cudaMemcpyAsync(c->h_err, B->d_errs, B->h_errs.size() * sizeof(int), cudaMemcpyDeviceToHost,
+                                    (cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "status words");
+    if ((e = cudaStreamSynchronize((cudaStream_t)stream)) != cudaSuccess) return cuda_fail(c, e, "stream synchronize");
+    memcpy(B->h_errs.data(), c->h_err, B->h_errs.size() * sizeof(int));
     const int job_rc = B->h_errs[0];
     bool attributed = false;
     for (int a = 0; a < B->n; a++) attributed |= B->h_errs[4 + a] != 0;
