@@ -38,11 +38,11 @@
 
 namespace acx {
 
-template <int NT>
+template <int NT, Loc kKind>
 __global__ void __launch_bounds__(NT, NT == kLocThreads ? 6 : NT == kLocWide ? 3 : 1) k_local(JobDev job) {
     extern __shared__ __align__(128) uint8_t sm[];
     grid_dependency_wait();  // the entropy stage's streams
-    local_worker<NT>(job, sm, 0, threadIdx.x);
+    local_worker<NT, kKind>(job, sm, 0, threadIdx.x);
 }
 
 // ---- cross-block pass --------------------------------------------------------------------
@@ -689,20 +689,27 @@ static int local_threads(size_t smem, uint32_t n_items, uint32_t T) {
     return 227 * 1024 / (smem + 1024) <= 4 ? kLocWide : kLocThreads;
 }
 
-template <int NT>
+template <int NT, Loc kKind>
 static cudaError_t local_attrs(size_t smem) {
-    cudaError_t e = cudaFuncSetAttribute(k_local<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_local<NT, kKind>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess)  // the whole unified L1 as shared memory: CTAs per SM are set by their workspaces
-        e = cudaFuncSetAttribute(k_local<NT>, cudaFuncAttributePreferredSharedMemoryCarveout,
+        e = cudaFuncSetAttribute(k_local<NT, kKind>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  cudaSharedmemCarveoutMaxShared);
     return e;
 }
 
+template <int NT, Loc kKind>
+static cudaError_t launch_local_kind(const JobDev& job, int grid, size_t smem, cudaStream_t st) {
+    const cudaError_t e = local_attrs<NT, kKind>(smem);
+    if (e != cudaSuccess) return e;
+    return launch_dependent(k_local<NT, kKind>, grid, NT, smem, st, job);
+}
 template <int NT>
 static cudaError_t launch_local_nt(const JobDev& job, int grid, size_t smem, cudaStream_t st) {
-    const cudaError_t e = local_attrs<NT>(smem);
-    if (e != cudaSuccess) return e;
-    return launch_dependent(k_local<NT>, grid, NT, smem, st, job);
+    // (a batch's archives have no item tables)
+    if (job.flags == 0 && !job.ready && job.arcs) return launch_local_kind<NT, Loc::kBatch>(job, grid, smem, st);
+    if (job.flags == 0 && !job.ready && !job.one.items) return launch_local_kind<NT, Loc::kOne>(job, grid, smem, st);
+    return launch_local_kind<NT, Loc::kAny>(job, grid, smem, st);
 }
 
 cudaError_t launch_local(const JobDev& job, int grid, cudaStream_t st) {
@@ -778,10 +785,10 @@ cudaError_t launch_external(const JobDev& job, int grid, cudaStream_t st) {
 }
 
 template <int NT>
-static int local_occupancy_nt(size_t smem) {
+static int local_occupancy_nt(size_t smem) {  // (all kinds are built for the same CTAs per SM)
     int n = 0;
-    if (local_attrs<NT>(smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_local<NT>, NT, smem) != cudaSuccess)
+    if (local_attrs<NT, Loc::kOne>(smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_local<NT, Loc::kOne>, NT, smem) != cudaSuccess)
         return 0;
     return n;
 }

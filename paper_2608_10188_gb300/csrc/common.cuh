@@ -151,6 +151,16 @@ struct ItemRef {
     uint32_t blk, slot, span_base, need_off, need_n;
     uint64_t scratch;
 };
+__device__ __forceinline__ ItemRef block_ref(const ArcJob& J, uint32_t idx) {  // (archives without an item table)
+    ItemRef r;
+    r.blk = J.lo + idx;
+    r.slot = r.blk;
+    r.need_off = 0;
+    r.need_n = 0;
+    r.span_base = J.blk[r.blk].span_base;
+    r.scratch = J.blk[r.blk].scratch;
+    return r;
+}
 __device__ __forceinline__ ItemRef item_ref(const ArcJob& J, uint32_t idx) {
     ItemRef r;
     if (J.items) {
@@ -162,12 +172,7 @@ __device__ __forceinline__ ItemRef item_ref(const ArcJob& J, uint32_t idx) {
         r.need_off = it.need_off;
         r.need_n = it.need_n;
     } else {
-        r.blk = J.lo + idx;
-        r.slot = r.blk;
-        r.need_off = 0;
-        r.need_n = 0;
-        r.span_base = J.blk[r.blk].span_base;
-        r.scratch = J.blk[r.blk].scratch;
+        r = block_ref(J, idx);
     }
     return r;
 }

@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(kFusedMaxThreads, 1) k_fused(JobDev job, int G
     }
     const int g = (warp - kFusedRansWarps) / kGroupWarps;
     if (g >= G) return;
-    local_worker<kLocThreads>(job, sm + F.loc + g * F.loc_stride, 1 + g, threadIdx.x - 32 * (kFusedRansWarps + kGroupWarps * g));
+    local_worker<kLocThreads, Loc::kAny>(job, sm + F.loc + g * F.loc_stride, 1 + g, threadIdx.x - 32 * (kFusedRansWarps + kGroupWarps * g));
 }
 
 int fused_groups(uint32_t max_tok, uint32_t max_lenb, uint32_t max_lit, bool lvl) {

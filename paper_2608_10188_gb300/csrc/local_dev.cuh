@@ -11,6 +11,21 @@ namespace acx {
 constexpr int kLocThreads = 128, kLocWide = 256, kLocWidest = 512;
 constexpr int kLocMaxWarps = kLocWidest / 32;
 
+// A loop of the local pass, rolled or left to the compiler.  Six CTAs of 128
+// threads, each at another point of the code, are limited by instruction
+// fetch, so their loops stay rolled (254 MB genome: 242 us, with the compiler's
+// unrolling 256); wider groups run longer loops on fewer blocks (200 MiB text: 447
+// and 421).
+template <bool kRolled, class F>
+__device__ __forceinline__ void each(uint32_t first, uint32_t end, uint32_t step, F f) {
+    if constexpr (kRolled) {
+#pragma unroll 1
+        for (uint32_t i = first; i < end; i += step) f(i);
+    } else {
+        for (uint32_t i = first; i < end; i += step) f(i);
+    }
+}
+
 struct LocLayout {
     uint32_t out, pend, tsrc, tpos, tll, tml, tlit, tcmd, tstat, lenb, soff, slit, scan, bar, misc, need, tlvl, tlvk,
         lhist, total;
@@ -89,7 +104,7 @@ __device__ __forceinline__ void block_scan(uint32_t (&v)[V], uint32_t (&tot)[V],
     uint32_t inc[V];
 #pragma unroll
     for (int k = 0; k < V; k++) inc[k] = v[k];
-#pragma unroll
+#pragma unroll(NT == kLocThreads ? 1 : 5)
     for (int o = 1; o < 32; o <<= 1) {
 #pragma unroll
         for (int k = 0; k < V; k++) {
@@ -158,18 +173,13 @@ __device__ __forceinline__ HMap hmap_compose(HMap f, HMap g) {
     return (uint64_t)(v[0] | (v[1] << 16)) | ((uint64_t)(v[2] | (v[3] << 16)) << 32);
 }
 
-__device__ __forceinline__ bool pend_clear_smem(const uint32_t* pend, uint32_t s, uint32_t e) {
-    if (s >= e) return true;
-    for (uint32_t w = s >> 5; w <= ((e - 1) >> 5); w++)
-        if (((volatile const uint32_t*)pend)[w] & range_mask(w, s, e)) return false;
-    return true;
-}
+template <bool kRolled>
 __device__ __forceinline__ void pend_update_smem(uint32_t* pend, uint32_t s, uint32_t e, bool set) {
     if (s >= e) return;
-    for (uint32_t w = s >> 5; w <= ((e - 1) >> 5); w++) {
+    each<kRolled>(s >> 5, ((e - 1) >> 5) + 1, 1, [&](uint32_t w) {
         const uint32_t m = range_mask(w, s, e);
         if (set) atomicOr(&pend[w], m); else atomicAnd(&pend[w], ~m);
-    }
+    });
 }
 
 // Run copy out[b, b+L) = src[a, a+L) (both in shared memory, the two ranges
@@ -179,25 +189,26 @@ __device__ __forceinline__ void pend_update_smem(uint32_t* pend, uint32_t s, uin
 // words may reach 3 bytes past the run, still inside the buffer (the literal
 // buffer is padded; a match source ends at or before its destination, which
 // holds at least 4 bytes); those bytes are shifted out unused.
+template <bool kRolled>
 __device__ __forceinline__ void copy_run8(uint8_t* sout, const uint8_t* lit, uint32_t a, uint32_t b, uint32_t L,
                                           uint32_t sl) {
     const uint32_t e = b + L;
     const uint32_t q0 = (b + 15) >> 4, q1 = e >> 4;  // whole 16-byte chunks [q0, q1)
     if (q0 >= q1) {
-        for (uint32_t x = b + sl; x < e; x += 8) sout[x] = lit[a + (x - b)];
+        each<kRolled>(b + sl, e, 8, [&](uint32_t x) { sout[x] = lit[a + (x - b)]; });
         return;
     }
-    for (uint32_t x = b + sl; x < 16 * q0; x += 8) sout[x] = lit[a + (x - b)];
-    for (uint32_t x = 16 * q1 + sl; x < e; x += 8) sout[x] = lit[a + (x - b)];
+    each<kRolled>(b + sl, 16 * q0, 8, [&](uint32_t x) { sout[x] = lit[a + (x - b)]; });
+    each<kRolled>(16 * q1 + sl, e, 8, [&](uint32_t x) { sout[x] = lit[a + (x - b)]; });
     const uint32_t* lw = reinterpret_cast<const uint32_t*>(lit);
     const uint32_t s0 = a + 16 * q0 - b;  // source of chunk q0
     const uint32_t sh = 8 * (s0 & 3);
-    for (uint32_t q = q0 + sl; q < q1; q += 8) {
+    each<kRolled>(q0 + sl, q1, 8, [&](uint32_t q) {
         const uint32_t w = (s0 >> 2) + 4 * (q - q0);
         const uint32_t x0 = lw[w], x1 = lw[w + 1], x2 = lw[w + 2], x3 = lw[w + 3], x4 = lw[w + 4];
         reinterpret_cast<uint4*>(sout)[q] = make_uint4(__funnelshift_r(x0, x1, sh), __funnelshift_r(x1, x2, sh),
                                                        __funnelshift_r(x2, x3, sh), __funnelshift_r(x3, x4, sh));
-    }
+    });
 }
 
 // Copy out[o, o + ml) = out[so, so + ml) (disjoint), by one thread: bytes up to
@@ -225,24 +236,45 @@ __device__ __forceinline__ void copy_lane(uint8_t* out, uint32_t so, uint32_t o,
 // Periodic fill out[o + k] = out[so + (k mod d)], k < ml, d < ml, by the eight
 // lanes sl of a lane group: it reads the period window [so, so + d) only, so
 // the lanes are independent; whole destination words as one store each.
+template <bool kRolled>
 __device__ __forceinline__ void fill_run8(uint8_t* out, uint32_t so, uint32_t o, uint32_t ml, uint32_t d, uint32_t sl) {
     const uint32_t e = o + ml, q0 = (o + 3) >> 2, q1 = e >> 2;  // whole words [q0, q1)
+    // k mod d with one division: k and d stay below 2^14 + 4, so the rounded-up
+    // reciprocal gives the quotient exactly
+    const uint32_t M = 0xffffffffu / d + 1;
+    auto mod = [&](uint32_t k) { return d == 1 ? 0u : k - d * __umulhi(k, M); };
     // ragged ends of at most 3 bytes: lanes 0..3 the head, 4..7 the tail
     const uint32_t edge = sl < 4 ? o + sl : max(4 * q1, 4 * q0) + sl - 4, edge_end = sl < 4 ? min(4 * q0, e) : e;
-    if (edge < edge_end) out[edge] = out[so + (edge - o) % d];
-    uint32_t r = (4 * (q0 + sl) - o) % d;
-    const uint32_t step = 32 % d;
-    for (uint32_t q = q0 + sl; q < q1; q += 8) {
-        uint32_t v = 0, x = r;
+    if (edge < edge_end) out[edge] = out[so + mod(edge - o)];
+    each<kRolled>(q0 + sl, q1, 8, [&](uint32_t q) {
+        uint32_t v = 0, x = mod(4 * q - o);
 #pragma unroll
         for (int u = 0; u < 4; u++) {
             v |= (uint32_t)out[so + x] << (8 * u);
             if (++x == d) x = 0;
         }
         reinterpret_cast<uint32_t*>(out)[q] = v;
-        r += step;
-        if (r >= d) r -= d;
-    }
+    });
+}
+
+// Plain copy out[o, o + ml) = out[so, so + ml) (disjoint), by the eight lanes sl
+// of a lane group: whole destination words from two source words each, bytes
+// at the ragged ends.  An in-block match is short (30 bytes on average in a
+// genome), where the 16-byte chunks of copy_run8 are mostly ragged ends.
+// Words may reach 3 bytes past the source run (never past the block: a source
+// ends at or before its destination).
+template <bool kRolled>
+__device__ __forceinline__ void copy_words8(uint8_t* out, uint32_t so, uint32_t o, uint32_t ml, uint32_t sl) {
+    const uint32_t e = o + ml, q0 = (o + 3) >> 2, q1 = e >> 2;  // whole words [q0, q1)
+    const uint32_t edge = sl < 4 ? o + sl : max(4 * q1, 4 * q0) + sl - 4, edge_end = sl < 4 ? min(4 * q0, e) : e;
+    if (edge < edge_end) out[edge] = out[so + edge - o];
+    const uint32_t* lw = reinterpret_cast<const uint32_t*>(out);
+    const uint32_t s0 = so + 4 * q0 - o, sh = 8 * (s0 & 3);
+    each<kRolled>(q0 + sl, q1, 8, [&](uint32_t q) {
+        const uint32_t w = (s0 >> 2) + q - q0;
+        const uint32_t x0 = lw[w], x1 = lw[w + 1];
+        reinterpret_cast<uint32_t*>(out)[q] = __funnelshift_r(x0, x1, sh);
+    });
 }
 
 // One pass by one warp over the listed in-block matches act[first + k],
@@ -261,7 +293,7 @@ __device__ __forceinline__ void fill_run8(uint8_t* out, uint32_t so, uint32_t o,
 // them (254 MB genome 318 -> 332 us; with G = 1 at every size 411).
 constexpr uint32_t kLaneCopy = 64;
 constexpr uint32_t kManyMatches = 64;  // more: G = 1
-template <uint32_t G>
+template <uint32_t G, bool kRolled>
 __device__ __forceinline__ uint32_t match_pass(const uint16_t* act, uint32_t n_act, uint32_t first, uint32_t stride,
                                                uint8_t* sout, uint32_t* pend, uint8_t* tstat, const uint16_t* tml,
                                                const uint16_t* tpos, const uint16_t* tll, const uint64_t* tsrc,
@@ -279,8 +311,9 @@ __device__ __forceinline__ uint32_t match_pass(const uint16_t* act, uint32_t n_a
             so = (uint32_t)(tsrc[i] - B);
             d = o - so;
             we = so + min(d, ml);  // periodic source window [so, we)
-            for (uint32_t w = (so >> 5) + sl; w <= ((we - 1) >> 5); w += G)
+            each<kRolled>((so >> 5) + sl, ((we - 1) >> 5) + 1, G, [&](uint32_t w) {
                 busy |= (((volatile uint32_t*)pend)[w] & range_mask(w, so, we)) != 0;
+            });
         }
         const uint32_t bm = __ballot_sync(ACX_FULL, busy);  // every lane, active or not
         const bool ready = on && (bm & gmask) == 0;
@@ -288,8 +321,8 @@ __device__ __forceinline__ uint32_t match_pass(const uint16_t* act, uint32_t n_a
         __threadfence_block();  // source reads after the readiness reads
         if (G == 8) {
             if (ready) {
-                if (d >= ml) copy_run8(sout, sout, so, o, ml, sl);
-                else fill_run8(sout, so, o, ml, d, sl);
+                if (d >= ml) copy_words8<kRolled>(sout, so, o, ml, sl);
+                else fill_run8<kRolled>(sout, so, o, ml, d, sl);
             }
         } else {
             const bool mine = ready && d >= ml && ml <= kLaneCopy;
@@ -305,16 +338,16 @@ __device__ __forceinline__ uint32_t match_pass(const uint16_t* act, uint32_t n_a
                 const uint32_t ml2 = __shfl_sync(ACX_FULL, ml, k & 31), o2 = __shfl_sync(ACX_FULL, o, k & 31),
                                so2 = __shfl_sync(ACX_FULL, so, k & 31);
                 if (k < 32) {
-                    if (o2 - so2 >= ml2) copy_run8(sout, sout, so2, o2, ml2, lane & 7);
-                    else fill_run8(sout, so2, o2, ml2, o2 - so2, lane & 7);
+                    if (o2 - so2 >= ml2) copy_words8<kRolled>(sout, so2, o2, ml2, lane & 7);
+                    else fill_run8<kRolled>(sout, so2, o2, ml2, o2 - so2, lane & 7);
                 }
             }
         }
         __syncwarp();
         __threadfence_block();
         if (ready) {
-            for (uint32_t w = (o >> 5) + sl; w <= ((o + ml - 1) >> 5); w += G)
-                atomicAnd(&pend[w], ~range_mask(w, o, o + ml));
+            each<kRolled>((o >> 5) + sl, ((o + ml - 1) >> 5) + 1, G,
+                          [&](uint32_t w) { atomicAnd(&pend[w], ~range_mask(w, o, o + ml)); });
             if (sl == 0) tstat[i] = 0;
             res |= 2;
         }
@@ -323,13 +356,37 @@ __device__ __forceinline__ uint32_t match_pass(const uint16_t* act, uint32_t n_a
     return res;
 }
 
+// The kind of job a local group is built for.  Whole decodes without levels
+// (one archive, or a batch of them: no wanted bytes, no level tables, no
+// parse-only records, no ready flags, no item tables) get code of their own:
+// the local pass loses issue slots to instruction fetch, and what such a job
+// never runs is as much again (254 MB genome 314 -> 290 us).
+enum class Loc { kAny, kOne, kBatch };
+template <Loc kKind>
+struct LocJob {
+    static constexpr bool kWhole = kKind != Loc::kAny;
+    static __device__ __forceinline__ bool flag(const JobDev& job, uint32_t f) { return !kWhole && (job.flags & f); }
+    static __device__ __forceinline__ bool fused(const JobDev& job) { return !kWhole && job.ready; }
+    static __device__ __forceinline__ int arc(const JobDev& job, uint32_t item) {
+        return kKind == Loc::kOne ? 0 : find_arc(job, item);
+    }
+    static __device__ __forceinline__ ArcJob load(const JobDev& job, int a) {
+        return kKind == Loc::kOne ? job.one : kKind == Loc::kBatch ? job.arcs[a] : load_arc(job, a);
+    }
+    static __device__ __forceinline__ ItemRef ref(const ArcJob& J, uint32_t idx) {
+        return kWhole ? block_ref(J, idx) : item_ref(J, idx);
+    }
+};
+
 // Issue the 1-D TMA copies of an item's four decoded streams (16-aligned,
 // padded) into the stream buffers (one thread).  Nothing is issued for a
 // block beyond the job's shared-memory limits (the caller treats it as bad).
+template <Loc kKind>
 __device__ __forceinline__ void stage_streams(const JobDev& job, uint32_t item, uint8_t* tcmd, uint8_t* lenb, uint8_t* soff,
                               uint8_t* slit, uint8_t* tlvl, uint64_t* bar) {
-    const ArcJob J = load_arc(job, find_arc(job, item));
-    const ItemRef ir = item_ref(J, item - J.item_base);
+    typedef LocJob<kKind> Kind;
+    const ArcJob J = Kind::load(job, Kind::arc(job, item));
+    const ItemRef ir = Kind::ref(J, item - J.item_base);
     const BlockDev& bd = J.blk[ir.blk];
     const uint32_t n = bd.n_tok, LB = bd.s_raw[kLen], n_new = bd.n_new, n_lit = bd.s_raw[kLit];
     if (n > job.max_tok || LB > job.max_lenb || n_new > job.max_tok || n_lit > job.max_lit) return;
@@ -337,7 +394,7 @@ __device__ __forceinline__ void stage_streams(const JobDev& job, uint32_t item, 
     const uint32_t sz[4] = {(n + 15) & ~15u, (LB + 15) & ~15u, (5 * n_new + 15) & ~15u, (n_lit + 15) & ~15u};
     uint8_t* dsts[4] = {tcmd, lenb, soff, slit};
     // the level body (stored in the payload, 16-aligned and padded) beside them
-    const uint32_t lsz = (job.flags & kJobLevels) && bd.lvl_body ? sz[0] : 0;
+    const uint32_t lsz = Kind::flag(job, kJobLevels) && bd.lvl_body ? sz[0] : 0;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // earlier generic use of the buffers
     mbar_arrive_tx(bar, sz[0] + sz[1] + sz[2] + sz[3] + lsz);
     for (int q = 0; q < 4; q++)
@@ -369,10 +426,12 @@ __device__ __forceinline__ bool wait_ready(const uint32_t* ready, uint32_t item,
 // The local pass of one group of NT threads (k_local: a whole CTA; k_fused: a
 // group of a fused CTA) over the job's tickets, with its workspace at sm and
 // named barrier bid; tid is the thread's index in its group.
-template <int NT>
+template <int NT, Loc kKind>
 __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uint32_t bid, int tid) {
-    const bool lvl = (job.flags & kJobLevels) != 0;
-    const LocLayout L = loc_layout(job.max_tok, job.max_lenb, job.max_lit, (job.flags & kJobNeed) != 0, lvl);
+    typedef LocJob<kKind> Kind;
+    constexpr bool kRolled = NT == kLocThreads;
+    const bool lvl = Kind::flag(job, kJobLevels);
+    const LocLayout L = loc_layout(job.max_tok, job.max_lenb, job.max_lit, Kind::flag(job, kJobNeed), lvl);
     uint8_t* tlvl = sm + L.tlvl;                                      // valid in kJobLevels jobs
     uint8_t* tlvk = sm + L.tlvk;
     uint32_t* lhist = reinterpret_cast<uint32_t*>(sm + L.lhist);
@@ -417,7 +476,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 cnext = misc[0];
                 cleft = chunk;
             }
-            item = ticket_item(job, cnext++);
+            item = Kind::kWhole ? cnext++ : ticket_item(job, cnext++);
             cleft--;
         }
         // the next block's ticket: its atomic goes out now and is read at the
@@ -436,9 +495,9 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             claimed = false;
         };
         if (item >= job.n_items) return;
-        const int a = find_arc(job, item);
-        const ArcJob J = load_arc(job, a);
-        const ItemRef ir = item_ref(J, item - J.item_base);
+        const int a = Kind::arc(job, item);
+        const ArcJob J = Kind::load(job, a);
+        const ItemRef ir = Kind::ref(J, item - J.item_base);
         const uint32_t b = ir.blk;
         const BlockDev& bd = J.blk[b];
         const uint64_t B = (uint64_t)b * kBlock;
@@ -452,12 +511,12 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
 
         // ---- stage the four decoded streams with 1-D TMA bulk copies (unless
         //      they were prefetched during the previous block) ----
-        if (!bad && tid == 0 && !prefetched && (!job.ready || wait_ready(job.ready, item, deadline)))
-            stage_streams(job, item, tcmd, lenb, soff, slit, tlvl, bar);
+        if (!bad && tid == 0 && !prefetched && (!Kind::fused(job) || wait_ready(job.ready, item, deadline)))
+            stage_streams<kKind>(job, item, tcmd, lenb, soff, slit, tlvl, bar);
         for (uint32_t i = tid; i < kBlock / 128; i += NT) reinterpret_cast<uint4*>(pend)[i] = make_uint4(0, 0, 0, 0);
         if (tid == 0) misc[1] = 0;
         // wanted bytes of this item (all when it names none)
-        const bool partial = (job.flags & kJobNeed) && ir.need_n != 0;
+        const bool partial = Kind::flag(job, kJobNeed) && ir.need_n != 0;
         if (partial) {
             for (uint32_t i = tid; i < kBlock / 32; i += NT) need[i] = 0;
             grp_sync<NT>(bid);
@@ -490,12 +549,12 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             uint32_t c = 0;
             bool vbad = false;
             if (!bad)
-                for (uint32_t j = j0; j < j1; j++) {
+                each<kRolled>(j0, j1, 1, [&](uint32_t j) {
                     const uint8_t by = lenb[j];
                     if (by < 0x80) c++;
                     // a value has at most three bytes
                     if (by >= 0x80 && j >= 2 && lenb[j - 1] >= 0x80 && lenb[j - 2] >= 0x80) vbad = true;
-                }
+                });
             if (vbad) misc[1] = 1;
             v1[0] = c;
             block_scan<NT, 1>(v1, tot1, scanbuf, bid, tid);
@@ -503,9 +562,9 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
         mark(tot1[0] != 2 * n || (LB > 0 && lenb[LB - 1] >= 0x80) || (LB == 0 && n > 0) || misc[1], kStageVarint);
         if (!bad) {
             uint32_t idx = v1[0];
-            for (uint32_t j = j0; j < j1; j++) {
+            each<kRolled>(j0, j1, 1, [&](uint32_t j) {
                 const uint8_t by = lenb[j];
-                if (by >= 0x80) continue;
+                if (by >= 0x80) return;
                 uint32_t val = by;
                 if (j >= 1 && lenb[j - 1] >= 0x80) {
                     val = (val << 7) | (lenb[j - 1] & 0x7f);
@@ -515,7 +574,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 const uint32_t tk = idx >> 1;
                 if (idx & 1) tml[tk] = (uint16_t)min(val, kBlock); else tll[tk] = (uint16_t)min(val, kBlock);
                 idx++;
-            }
+            });
         }
         grp_sync<NT>(bid);
         mark(misc[1] != 0, kStageVarint);
@@ -528,7 +587,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             uint32_t s_len = 0, s_ll = 0, s_new = 0;
             bool tbad = false;
             if (!bad)
-                for (uint32_t i = i0; i < i1; i++) {
+                each<kRolled>(i0, i1, 1, [&](uint32_t i) {
                     const uint32_t ll = tll[i], ml = tml[i], c = tcmd[i];
                     s_len += ll + ml;
                     s_ll += ll;
@@ -537,7 +596,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                     if (c == kLitOnly) { if (ml != 0 || i != n - 1 || ll == 0) tbad = true; }
                     else if (ml < J.min_match) tbad = true;
                     any_rep |= c >= 1 && c <= 4;
-                }
+                });
             if (tbad) misc[1] = 1;
             v3[0] = s_len; v3[1] = s_ll; v3[2] = s_new;
             block_scan<NT, 3>(v3, tot3, scanbuf, bid, tid);
@@ -545,7 +604,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
         mark(tot3[0] != R || tot3[1] != n_lit || tot3[2] != n_new || misc[1], kStageTokens);
         if (!bad) {
             uint32_t pos = v3[0], lp = v3[1], ni = v3[2];
-            for (uint32_t i = i0; i < i1; i++) {
+            each<kRolled>(i0, i1, 1, [&](uint32_t i) {
                 const uint32_t ll = tll[i], ml = tml[i];
                 tpos[i] = (uint16_t)pos;
                 tlit[i] = (uint16_t)lp;
@@ -559,7 +618,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 tsrc[i] = src;
                 pos += ll + ml;
                 lp += ll;
-            }
+            });
         }
         any_rep = grp_or<NT>(bid, any_rep && !bad);
         mark(misc[1] != 0, kStageSources);
@@ -568,16 +627,16 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
         //      warp-level scan of packed maps by warp 0, while the other warps
         //      place the literals, which need positions only (a parse-only job
         //      places none) ----
-        const bool place = !bad && !(job.flags & kJobIndex);
+        const bool place = !bad && !Kind::flag(job, kJobIndex);
         if (!bad && (any_rep || place)) {
             if (any_rep && warp == 0) {
                 const uint32_t per = (n + 31) / 32;
                 const uint32_t j0 = min(n, lane * per), j1 = min(n, j0 + per);
                 HMap agg = kHIdentity;
-                for (uint32_t i = j0; i < j1; i++) agg = hmap_step(agg, tcmd[i], i);
+                each<kRolled>(j0, j1, 1, [&](uint32_t i) { agg = hmap_step(agg, tcmd[i], i); });
                 // inclusive scan of the lanes' maps (earlier maps act first)
                 HMap inc = agg;
-#pragma unroll
+#pragma unroll 1
                 for (int o = 1; o < 32; o <<= 1) {
                     const HMap prev = __shfl_up_sync(ACX_FULL, inc, o);
                     if (lane >= o) inc = hmap_compose(prev, inc);
@@ -592,7 +651,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 };
                 // the lane's history in four registers (selects, no indexed array)
                 uint64_t h0 = entry(0), h1 = entry(1), h2 = entry(2), h3 = entry(3);
-                for (uint32_t i = j0; i < j1; i++) {
+                each<kRolled>(j0, j1, 1, [&](uint32_t i) {
                     const uint8_t c = tcmd[i];
                     const uint64_t dst = B + tpos[i] + tll[i];
                     if (c == kNew) {
@@ -607,12 +666,13 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                         h1 = j >= 1 ? h0 : h1;
                         h0 = d;
                     }
-                }
+                });
             }
             if (place && (warp > 0 || !any_rep)) {
                 // literal placement: a thread copies a tiny run (<= kLaneBytes)
                 // by itself, all threads at once; eight lanes copy each longer one
                 const int w0 = any_rep ? 1 : 0, nw = (NT / 32) - w0;
+#pragma unroll 1
                 for (uint32_t i = tid - 32 * w0; i < n; i += 32 * nw) {
                     const uint32_t ll = tll[i];
                     if (ll <= kLaneBytes) {
@@ -620,8 +680,9 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                         for (uint32_t k = 0; k < ll; k++) sout[lb + k] = slit[la + k];
                     }
                 }
+#pragma unroll 1
                 for (uint32_t i = (warp - w0) * 4 + (lane >> 3); i < n; i += nw * 4)
-                    if (tll[i] > kLaneBytes) copy_run8(sout, slit, tlit[i], tpos[i], tll[i], lane & 7);
+                    if (tll[i] > kLaneBytes) copy_run8<kRolled>(sout, slit, tlit[i], tpos[i], tll[i], lane & 7);
             }
             grp_sync<NT>(bid);
             mark(misc[1] != 0, kStageSources);
@@ -646,7 +707,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             mark(misc[1] != 0, kStageSources);
         }
 
-        if (job.flags & kJobIndex) {
+        if (Kind::flag(job, kJobIndex)) {
             // parse only: one record per token (source, destination offset,
             // match length, command)
             if (!bad)
@@ -669,12 +730,13 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             uint16_t* act_list = tlit;
             if (tid == 0) misc[3] = 0;
             grp_sync<NT>(bid);
+#pragma unroll 1
             for (uint32_t i = tid; i < n; i += NT) {
                 const uint32_t ml = tml[i];
                 uint8_t st = 0;  // 0: none/done, 1: unresolved in-block, 2: pending
                 if (ml) {
                     const uint32_t s = tpos[i] + tll[i];
-                    pend_update_smem(pend, s, s + ml, true);
+                    pend_update_smem<kRolled>(pend, s, s + ml, true);
                     st = tsrc[i] >= B ? 1 : 2;
                     if (st == 1) act_list[atomicAdd((uint32_t*)&misc[3], 1u)] = (uint16_t)i;
                 }
@@ -685,17 +747,17 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             // ---- the stream buffers are free from here on: start the next item's
             //      copies, so that they land while this block finishes ----
             settle_claim();
-            pf_item = ticket_item(job, cnext++);
+            pf_item = Kind::kWhole ? cnext++ : ticket_item(job, cnext++);
             cleft--;
             // (issued by the last warp, which takes the fewest in-block matches
             // below, so that its loads of the next block's descriptor delay the
             // rounds least)
             if (tid == NT - 32) {
                 // in a fused decode, only streams that are already published
-                const bool go = pf_item < job.n_items && (!job.ready || ld_acquire_u32(job.ready + pf_item) != 0);
+                const bool go = pf_item < job.n_items && (!Kind::fused(job) || ld_acquire_u32(job.ready + pf_item) != 0);
                 if (go) {
-                    if (job.ready) asm volatile("fence.proxy.async.global;" ::: "memory");
-                    stage_streams(job, pf_item, tcmd, lenb, soff, slit, tlvl, bar);
+                    if (Kind::fused(job)) asm volatile("fence.proxy.async.global;" ::: "memory");
+                    stage_streams<kKind>(job, pf_item, tcmd, lenb, soff, slit, tlvl, bar);
                 }
                 misc[2] = go;
             }
@@ -704,8 +766,8 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             for (;;) {
                 const uint32_t r =
                     NT > kLocThreads && n_act > kManyMatches
-                        ? match_pass<1>(tlit, n_act, 32 * warp, NT, sout, pend, tstat, tml, tpos, tll, tsrc, B, lane)
-                        : match_pass<8>(tlit, n_act, 4 * warp, NT / 8, sout, pend, tstat, tml, tpos, tll, tsrc, B, lane);
+                        ? match_pass<1, kRolled>(tlit, n_act, 32 * warp, NT, sout, pend, tstat, tml, tpos, tll, tsrc, B, lane)
+                        : match_pass<8, kRolled>(tlit, n_act, 4 * warp, NT / 8, sout, pend, tstat, tml, tpos, tll, tsrc, B, lane);
                 const int any_left = grp_or<NT>(bid, r & 1);
                 const int any_prog = grp_or<NT>(bid, r & 2);
                 if (!any_left || !any_prog) break;
@@ -713,9 +775,11 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             // ---- whatever is still unresolved becomes pending pieces (for a
             //      partial item: the wanted matches only) ----
             if (partial)
+#pragma unroll 1
                 for (uint32_t i = i0; i < i1; i++)
                     if (tstat[i] && !wanted(need, tpos[i] + tll[i], tml[i])) tstat[i] = 0;
             uint32_t cnt = 0, nbytes = 0;
+#pragma unroll 1
             for (uint32_t i = i0; i < i1; i++)
                 if (tstat[i]) {
                     cnt += pieces_of(tml[i]);
@@ -755,6 +819,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             }
             {
                 uint32_t k = v2[0];
+#pragma unroll 1
                 for (uint32_t i = i0; i < i1; i++) {
                     if (!tstat[i]) continue;
                     const uint32_t o = tpos[i] + tll[i];
@@ -775,6 +840,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
         uint8_t* gout = J.out + (uint64_t)ir.slot * kBlock;
         const uint32_t nv = R / 16;
         for (uint32_t i = tid; i < nv; i += NT) reinterpret_cast<uint4*>(gout)[i] = reinterpret_cast<uint4*>(sout)[i];
+#pragma unroll 1
         for (uint32_t x = 16 * nv + tid; x < R; x += NT) gout[x] = sout[x];
         {
             // the pending bitmap is written for every block (all clear when nothing

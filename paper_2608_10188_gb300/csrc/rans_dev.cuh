@@ -57,7 +57,7 @@ struct TabLoad {
     uint64_t* bar;
     uint32_t phase;
 };
-__device__ __forceinline__ bool wait_table(const TabLoad& T, int s, uint64_t deadline) {
+__device__ __forceinline__ bool wait_table(TabLoad T, int s, uint64_t deadline) {
     if (!T.bar) return true;
     uint32_t spins = 0;
     bool ok = true;
@@ -114,7 +114,7 @@ __device__ __forceinline__ void rans_renorm(uint32_t& x, uint32_t& rb, uint32_t 
 // mbarrier phase bookkeeping across streams).  Returns false on a format
 // violation (word overrun, end states != 2^16) or an expired wait.
 template <int S>
-__device__ __forceinline__ bool rans_stream(const TabLoad& T, int type, uint32_t tab_s, const uint8_t* __restrict__ body, uint32_t enc,
+__device__ __forceinline__ bool rans_stream(TabLoad T, int type, uint32_t tab_s, const uint8_t* __restrict__ body, uint32_t enc,
                                             uint32_t n, uint32_t K, uint8_t* __restrict__ out, uint32_t ring_s,
                                             uint32_t stage_s, uint64_t* bar, uint32_t& seq, int lane,
                                             uint64_t deadline) {
@@ -233,12 +233,12 @@ __device__ __forceinline__ bool rans_stream(const TabLoad& T, int type, uint32_t
 // The wide-lane variants are rare (archives encoded with more than 32
 // lanes): out of line, so that they do not raise the kernel's register
 // pressure.
-static __device__ __noinline__ bool rans_stream2(const TabLoad& T, int type, uint32_t tab_s, const uint8_t* body, uint32_t enc, uint32_t n, uint32_t K,
+static __device__ __noinline__ bool rans_stream2(TabLoad T, int type, uint32_t tab_s, const uint8_t* body, uint32_t enc, uint32_t n, uint32_t K,
                                           uint8_t* out, uint32_t ring_s, uint32_t stage_s, uint64_t* bar,
                                           uint32_t& seq, int lane, uint64_t deadline) {
     return rans_stream<2>(T, type, tab_s, body, enc, n, K, out, ring_s, stage_s, bar, seq, lane, deadline);
 }
-static __device__ __noinline__ bool rans_stream4(const TabLoad& T, int type, uint32_t tab_s, const uint8_t* body, uint32_t enc, uint32_t n, uint32_t K,
+static __device__ __noinline__ bool rans_stream4(TabLoad T, int type, uint32_t tab_s, const uint8_t* body, uint32_t enc, uint32_t n, uint32_t K,
                                           uint8_t* out, uint32_t ring_s, uint32_t stage_s, uint64_t* bar,
                                           uint32_t& seq, int lane, uint64_t deadline) {
     return rans_stream<4>(T, type, tab_s, body, enc, n, K, out, ring_s, stage_s, bar, seq, lane, deadline);
@@ -269,7 +269,7 @@ __device__ __forceinline__ uint32_t short_group(const BlockDev& bd) {
 // warp: stream g runs on lanes [lo_g, lo_g + K_g) with its own word pointer;
 // their words are staged whole into the warp's ring by TMA.  Returns false on
 // a format violation or an expired wait.
-__device__ __forceinline__ bool rans_short(const TabLoad& T, uint32_t mask, uint32_t tab0_s, const BlockDev& bd, const uint8_t* pay,
+__device__ __forceinline__ bool rans_short(TabLoad T, uint32_t mask, uint32_t tab0_s, const BlockDev& bd, const uint8_t* pay,
                                            uint8_t* scr, uint32_t ring_s, uint64_t* sbar, uint32_t& sphase, int lane,
                                            uint64_t deadline) {
     uint32_t lo[3], K[3], W[3], hdr[3], roff[3], nw_bytes[3];
@@ -380,7 +380,7 @@ constexpr uint32_t kRansParts = 3, kRansAll = 3;
 // 16-aligned) are the warp's own.  A corrupt stream sets the job's (and the
 // archive's) error status.
 __device__ __forceinline__ void rans_block(const JobDev& job, int a, const ArcJob& J, const ItemRef& ir,
-                                           uint32_t part, const TabLoad& T, uint32_t tab0_s, uint32_t ring_s, uint32_t stage_s,
+                                           uint32_t part, TabLoad T, uint32_t tab0_s, uint32_t ring_s, uint32_t stage_s,
                                            uint64_t* bar, uint64_t* sbar, uint32_t& seq, uint32_t& sphase, int lane,
                                            uint64_t deadline) {
     const uint32_t b = ir.blk;
