@@ -28,7 +28,10 @@ __global__ void k_prologue(uint32_t* counters, uint32_t n_counters, int* errs, u
 // Each CTA works on one archive at a time (its tables in shared memory);
 // its warps take blocks of that archive from the archive's ticket, and when
 // the archive is exhausted the CTA moves to the archive with the most blocks
-// left.
+// left.  A lone archive has a kernel of its own, which reads its job from the
+// parameters: with the archive's fields in registers the kernel, at its 64 per
+// thread, spilled four times as much (254 MB genome 254 -> 240 us).
+template <bool kMulti>
 __global__ void __launch_bounds__(kRansWarps * 32) k_rans(JobDev job) {
     extern __shared__ __align__(128) uint8_t smraw[];
     RansSmem& S = *reinterpret_cast<RansSmem*>(smraw);
@@ -40,7 +43,7 @@ __global__ void __launch_bounds__(kRansWarps * 32) k_rans(JobDev job) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if (threadIdx.x == 0) {
         const uint64_t target = (uint64_t)blockIdx.x * job.n_items / gridDim.x;
-        S.next_arc = job.n_arcs > 1 ? find_arc(job, (uint32_t)target) : 0;
+        S.next_arc = kMulti ? find_arc(job, (uint32_t)target) : 0;
         S.arc = -1;
     }
     __syncthreads();
@@ -51,7 +54,7 @@ __global__ void __launch_bounds__(kRansWarps * 32) k_rans(JobDev job) {
     for (;;) {
         const int a = S.next_arc;
         if (a < 0) break;
-        const ArcJob J = load_arc(job, a);
+        const ArcJob J = kMulti ? job.arcs[a] : job.one;
         if (S.arc != a) {
             // (every warp has left the tables of the archive before)
             if (threadIdx.x == 0) {
@@ -77,7 +80,7 @@ __global__ void __launch_bounds__(kRansWarps * 32) k_rans(JobDev job) {
         // the work starts spread over the SMs however their CTAs come up
         const uint32_t n_blk = J.hi - J.lo, n_a = n_blk * job.rans_parts;
         const uint32_t chunk = job.chunk ? job.chunk : 1u;
-        const uint32_t own = job.n_arcs == 1 ? gridDim.x * kRansWarps * chunk : 0u;
+        const uint32_t own = kMulti ? 0u : gridDim.x * kRansWarps * chunk;
         uint32_t cnext = (warp * gridDim.x + blockIdx.x) * chunk;  // this warp's current run of `chunk` tickets
         uint32_t cleft = own ? chunk : 0u;
         for (;;) {
@@ -99,7 +102,7 @@ __global__ void __launch_bounds__(kRansWarps * 32) k_rans(JobDev job) {
         // before the CTA leaves or the next archive's go out
         if (warp == 0)
             for (int s = 0; s < 4; s++) wait_table(T, s, deadline);
-        if (job.n_arcs == 1) break;
+        if (!kMulti) break;
         __syncthreads();
         if (warp == 0) {
             // the archive with the most tickets left, the lowest of equals
@@ -139,7 +142,8 @@ cudaError_t launch_prologue(uint32_t* counters, uint32_t n_counters, cudaStream_
 cudaError_t launch_rans(const JobDev& job_in, int grid, cudaStream_t st) {
     JobDev job = job_in;
     const size_t sm = rans_smem_bytes();
-    cudaError_t e = cudaFuncSetAttribute(k_rans, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const auto kernel = job.arcs ? k_rans<true> : k_rans<false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     // When every part of every block finds a warp at once, a block's streams
     // decode on three warps and only the longest counts (one 10 KB text block
@@ -153,15 +157,18 @@ cudaError_t launch_rans(const JobDev& job_in, int grid, cudaStream_t st) {
     const uint64_t per_cta = (uint64_t)kRansWarps * (job.chunk ? job.chunk : 1);
     const uint64_t need = ((uint64_t)job.n_items * job.rans_parts + per_cta - 1) / per_cta;
     if (need <= (uint64_t)noted_sm_count()) grid = std::min(grid, noted_sm_count());
-    return launch_dependent(k_rans, grid, kRansWarps * 32, sm, st, job);
+    return launch_dependent(kernel, grid, kRansWarps * 32, sm, st, job);
 }
 
 int rans_occupancy() {
     const size_t sm = rans_smem_bytes();
-    cudaFuncSetAttribute(k_rans, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_rans, kRansWarps * 32, sm) != cudaSuccess) return 0;
-    return n;
+    int n = 0, m = 0;
+    cudaFuncSetAttribute(k_rans<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(k_rans<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_rans<false>, kRansWarps * 32, sm) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, k_rans<true>, kRansWarps * 32, sm) != cudaSuccess)
+        return 0;
+    return std::min(n, m);
 }
 
 }  // namespace acx
