@@ -38,8 +38,15 @@
 
 namespace acx {
 
+// CTAs per SM that the registers allow.  A lone archive of large blocks (55 KB of
+// workspace) has four of 256 threads, at 61 registers (200 MiB text: three 423
+// us, four 357); a batch's kernel loses more to spills than the fourth gives (646
+// us for 96 files, 657 with it).
 template <int NT, Loc kKind>
-__global__ void __launch_bounds__(NT, NT == kLocThreads ? 6 : NT == kLocWide ? 3 : 1) k_local(JobDev job) {
+constexpr int kLocCtas = NT == kLocThreads ? 6 : NT == kLocWidest ? 1 : kKind == Loc::kOne ? 4 : 3;
+
+template <int NT, Loc kKind>
+__global__ void __launch_bounds__(NT, kLocCtas<NT, kKind>) k_local(JobDev job) {
     extern __shared__ __align__(128) uint8_t sm[];
     grid_dependency_wait();  // the entropy stage's streams
     local_worker<NT, kKind>(job, sm, 0, threadIdx.x);
@@ -678,8 +685,8 @@ size_t local_smem_bytes(uint32_t T, uint32_t LB, uint32_t LIT, bool need, bool l
 // Threads of a local CTA for a job of n_items blocks of up to T tokens whose
 // workspace has `smem` bytes.  A CTA's shared memory sets how many fit an SM:
 // with four or fewer (blocks of some 900 tokens and more), 128 threads leave
-// most of the SM's issue slots empty (200 MiB text: 487 us; 256 threads 461; a
-// batch of 96 files 936 -> 825), with five or six they fill it (254 MB genome:
+// most of the SM's issue slots empty (200 MiB text: 487 us; 256 threads 461, and
+// 357 since four of them fit; a batch of 96 files 936 -> 825), with five or six they fill it (254 MB genome:
 // 322 us; 256 threads 420).  A job of few blocks has every block on an SM at
 // once, so only a block's latency counts: 256 threads, or 512 for blocks of
 // many tokens (4 MiB DNA-like 34 -> 27 us; 4 MiB text 97 -> 73 -> 60 with 128,
@@ -785,7 +792,7 @@ cudaError_t launch_external(const JobDev& job, int grid, cudaStream_t st) {
 }
 
 template <int NT>
-static int local_occupancy_nt(size_t smem) {  // (all kinds are built for the same CTAs per SM)
+static int local_occupancy_nt(size_t smem) {  // (of the kind that runs most CTAs: a grid may exceed what is resident)
     int n = 0;
     if (local_attrs<NT, Loc::kOne>(smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_local<NT, Loc::kOne>, NT, smem) != cudaSuccess)
