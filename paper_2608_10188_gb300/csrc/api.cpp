@@ -464,11 +464,15 @@ int aceapex_decode_all(aceapex_ctx* c, aceapex_archive* A, void* d_out, uint64_t
 // output is downloaded on a third stream while chunk k + 1 decodes.  A
 // chunk's cross-block sources lie in its own or earlier blocks (every source
 // precedes its destination), all final when its decode runs.  The download
-// is the slowest leg (the host link carries about 190 GB/s, the decode about
-// 280), so the first chunk is small, to start it early, and the later ones
-// large, to keep the per-launch costs of the decode low.
+// is the slowest leg (the host link carries about 190 GB/s, the decode up to
+// 400), so the first chunk is smaller than the later ones, to start it early.
+// It isn't smaller still: a chunk of 512 blocks leaves most of the device idle
+// and costs three launches and their tails for 8 MiB.  Measured on DNA-like
+// data with a first chunk of 1536 blocks, and before with 512 and 1536: 16 MiB
+// 286 us (343), 28 MiB 380 (428), 64 MiB 610 (642), 100 MiB 849 (900), 242 MiB
+// 1634 (1680); 64 MiB text 904 (897); 2048 first is the same within 1%.
 static uint32_t host_chunk_end(uint32_t lo, uint32_t n_blocks) {
-    const uint32_t hi = lo == 0 ? 512 : lo < 2048 ? 2048 : lo + 4096;
+    const uint32_t hi = lo == 0 ? 1536 : lo + 4096;
     return std::min(hi, n_blocks);
 }
 

@@ -1,5 +1,5 @@
 """End-to-end decode from host memory (aceapex_decode_host), a pipeline over
-chunks of blocks (512, 1536, then 4096 each): uploads, chunk decodes and
+chunks of blocks (1536, then 4096 each): uploads, chunk decodes and
 downloads on three streams.  Archives of one chunk, several chunks and a
 ragged last chunk decode to the oracle's bytes, with and without
 level-ordered cross-block passes, history and history-free, on an opened
@@ -27,9 +27,11 @@ def acx():
 
 
 @pytest.mark.parametrize("kind,size,kw", [
-    ("dna", 6144 * BLOCK + 5 * BLOCK + 123, {}),                      # 4 chunks, ragged last one
-    ("text", 2048 * BLOCK + 77, {"levels": True}),                    # 3 chunks, level order
-    ("dna", 512 * BLOCK, {"no_rep": True}),                           # exactly one chunk
+    ("dna", 6144 * BLOCK + 5 * BLOCK + 123, {}),                      # 3 chunks, ragged last one
+    ("text", 2048 * BLOCK + 77, {"levels": True}),                    # 2 chunks, level order
+    ("dna", 512 * BLOCK, {"no_rep": True}),                           # one chunk
+    ("dna", 1536 * BLOCK, {}),                                        # exactly one chunk
+    ("dna", 1536 * BLOCK + 1, {}),                                    # and one byte more
     ("text", 100_000, {"no_rep": True, "levels": True}),              # less than a chunk
 ])
 def test_host_pipeline_matches_oracle(acx, kind, size, kw):
