@@ -465,14 +465,17 @@ int aceapex_decode_all(aceapex_ctx* c, aceapex_archive* A, void* d_out, uint64_t
 // chunk's cross-block sources lie in its own or earlier blocks (every source
 // precedes its destination), all final when its decode runs.  The download
 // is the slowest leg (the host link carries about 190 GB/s, the decode up to
-// 400), so the first chunk is smaller than the later ones, to start it early.
-// It isn't smaller still: a chunk of 512 blocks leaves most of the device idle
-// and costs three launches and their tails for 8 MiB.  Measured on DNA-like
-// data with a first chunk of 1536 blocks, and before with 512 and 1536: 16 MiB
-// 286 us (343), 28 MiB 380 (428), 64 MiB 610 (642), 100 MiB 849 (900), 242 MiB
-// 1634 (1680); 64 MiB text 904 (897); 2048 first is the same within 1%.
+// 400), so it has to start early and the decode has to stay ahead of it: a
+// first chunk of 1536 blocks, then 2048 each.  The first isn't smaller: a chunk
+// of 512 blocks leaves most of the device idle and costs three launches and
+// their tails for 8 MiB.  The later ones aren't larger: the last chunk's download
+// runs alone, and text decodes no faster than the link.  Measured (with 512, 1536,
+// then 4096 each | 1536, then 4096 | 1536, then 1536), DNA-like data: 16 MiB 287
+// us (343 | 286 | 287), 28 MiB 382 (428 | 381 | 382), 64 MiB 605 (642 | 612 |
+// 597), 100 MiB 787 (900 | 844 | 778), 242 MiB 1621 (1680 | 1634 | 1648); text:
+// 64 MiB 829 (897 | 882 | 810), 128 MiB 1333 (1412 | 1341 | 1318).
 static uint32_t host_chunk_end(uint32_t lo, uint32_t n_blocks) {
-    const uint32_t hi = lo == 0 ? 1536 : lo + 4096;
+    const uint32_t hi = lo == 0 ? 1536 : lo + 2048;
     return std::min(hi, n_blocks);
 }
 

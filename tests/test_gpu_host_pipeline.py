@@ -1,5 +1,5 @@
 """End-to-end decode from host memory (aceapex_decode_host), a pipeline over
-chunks of blocks (1536, then 4096 each): uploads, chunk decodes and
+chunks of blocks (1536, then 2048 each): uploads, chunk decodes and
 downloads on three streams.  Archives of one chunk, several chunks and a
 ragged last chunk decode to the oracle's bytes, with and without
 level-ordered cross-block passes, history and history-free, on an opened
@@ -27,7 +27,7 @@ def acx():
 
 
 @pytest.mark.parametrize("kind,size,kw", [
-    ("dna", 6144 * BLOCK + 5 * BLOCK + 123, {}),                      # 3 chunks, ragged last one
+    ("dna", 6144 * BLOCK + 5 * BLOCK + 123, {}),                      # 4 chunks, ragged last one
     ("text", 2048 * BLOCK + 77, {"levels": True}),                    # 2 chunks, level order
     ("dna", 512 * BLOCK, {"no_rep": True}),                           # one chunk
     ("dna", 1536 * BLOCK, {}),                                        # exactly one chunk
