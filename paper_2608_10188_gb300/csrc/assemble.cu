@@ -1,7 +1,7 @@
 // Parse and match layer of the decode (paper: "parse" and "copy"), in two
 // passes separated by a kernel boundary.
 //
-// k_local (one CTA of 128 threads per block, persistent, any order):
+// k_local (one CTA of 128, 256 or 512 threads per block, persistent, any order):
 //   * varint boundaries by compaction: every byte < 0x80 ends a value; a CTA
 //     prefix count gives each value its index (LL_i, ML_i).  The paper finds
 //     varints make 0.61% of commands sequential in a serial parse ("The Last
@@ -14,14 +14,15 @@
 //     prefix "sum" too.  Skipped when a block has no repeat code (history-
 //     free encoding, where the parse is a dependency-free prefix scan).
 //   * literals: runs of up to 32 bytes are copied by one thread each, all
-//     threads at once; longer runs by a warp with 4-byte funnel-shifted copies.
+//     threads at once; longer runs by eight lanes with 16-byte funnel-shifted
+//     stores.
 //   * matches whose source lies inside the block are periodic fills
 //     out[dst+k] = out[src + (k mod d)] ("What Does: Periods, Not Chains"),
 //     done in rounds as their sources become final; matches whose source
 //     chain leaves the block become pending spans.
 //   * the block is written with coalesced 16-byte stores; its pending-byte
 //     bitmap and pending spans go beside it.
-// k_external (warps take parts of blocks in ascending order, one lane per span):
+// k_external (warps take parts of blocks in ascending order, a lane per span):
 //   after the kernel boundary every literal and every in-block match byte is
 //   final, so a pending span waits only on the spans its source really
 //   depends on, which lie at lower positions and were taken earlier: the
@@ -100,9 +101,9 @@ constexpr int kExtThreads = 1024;
 // flight at once, so that chains between them clog the lanes; in parts, the
 // pieces in flight are a narrow window of the output, and a wait without limit
 // pays at every size.  Zipf text: 1 MiB 195 -> 35 us, 4 MiB 238 -> 55, 16 MiB
-// 242 -> 82, 64 MiB 418 -> 297, 200 MiB 1091 (in level order) -> 760; DNA-like
-// 4 MiB 43 -> 34, 64 MiB 70 -> 59.  With parts of 32 / 128 pieces the 200 MiB text takes
-// 881 / 832 us, and DNA-like 64 MiB 61 / 72.
+// 242 -> 82, 64 MiB 418 -> 295, 200 MiB 1091 (in level order) -> 750; DNA-like
+// 4 MiB 43 -> 34, 64 MiB 70 -> 59.  With parts of 32 / 48 / 96 / 128 pieces the
+// 200 MiB text takes 881 / 772 / 758 / 832 us, and DNA-like 64 MiB 61 / 59 / 74 / 72.
 constexpr uint32_t kPartPieces = 64;
 
 // Are the bytes a piece reads final?  (period 0: [src, src+len); otherwise the

@@ -14,8 +14,8 @@ constexpr int kLocMaxWarps = kLocWidest / 32;
 // A loop of the local pass, rolled or left to the compiler.  Six CTAs of 128
 // threads, each at another point of the code, are limited by instruction
 // fetch, so their loops stay rolled (254 MB genome: 242 us, with the compiler's
-// unrolling 256); wider groups run longer loops on fewer blocks (200 MiB text: 447
-// and 421).
+// unrolling 256); wider groups run longer loops on fewer blocks (200 MiB text, at
+// three CTAs per SM: 447 and 421).
 template <bool kRolled, class F>
 __device__ __forceinline__ void each(uint32_t first, uint32_t end, uint32_t step, F f) {
     if constexpr (kRolled) {
