@@ -552,7 +552,8 @@ def run_batch(args, dist):
             "cross_block_stats": {"pending_pieces": sst.get("pending_spans"), "pending_bytes": sst.get("pending_bytes"),
                                   "rounds_after_first": sst.get("wait_polls")},
             "roofline": roof, "path_roofline": path_roof, "e2e": None, "cpu_baseline": cpu,
-            "gpu_launches": 4 * args.steps, "clocks": clk,
+            "gpu_launches": 4 * args.steps,  # at least: a large batch of two kinds has a second local pass
+            "clocks": clk,
         }
         print(json.dumps(line), flush=True)
     B.close()

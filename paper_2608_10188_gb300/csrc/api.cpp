@@ -376,7 +376,20 @@ int acx::enqueue_job(aceapex_ctx* c, const JobDev& job_in, const LaunchPlan& lp,
     } else if (lp.variant == ACEAPEX_VARIANT_PLAIN) {
         if ((e = launch_plain(job, lp.grid_plain, st)) != cudaSuccess) return cuda_fail(c, e, "plain launch");
     } else {
-        if ((e = launch_local(job, lp.grid_local, st)) != cudaSuccess) return cuda_fail(c, e, "local launch");
+        const bool split = job.cls[0].items != 0;
+        for (uint32_t k = 0; k < (split ? 2u : 1u); k++) {
+            JobDev j = job;
+            if (split) {
+                j.max_tok = job.cls[k].max_tok;
+                j.max_lenb = job.cls[k].max_lenb;
+                j.max_lit = job.cls[k].max_lit;
+                j.loc_lo = k ? job.cls[0].items : 0;
+                j.loc_hi = j.loc_lo + job.cls[k].items;
+                j.loc_ctr = k ? 0 : 1;
+            }
+            if ((e = launch_local(j, split ? lp.grid_cls[k] : lp.grid_local, st)) != cudaSuccess)
+                return cuda_fail(c, e, "local launch");
+        }
     }
     if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return cuda_fail(c, e, "event");
     if ((job.flags & kJobLevels) && (e = launch_level_list(job, st)) != cudaSuccess)

@@ -39,15 +39,16 @@
 
 namespace acx {
 
-// CTAs per SM that the registers allow.  A lone archive of large blocks (55 KB of
-// workspace) has four of 256 threads, at 61 registers (200 MiB text: three 423
-// us, four 357); a batch's kernel loses more to spills than the fourth gives (646
-// us for 96 files, 657 with it).
-template <int NT, Loc kKind>
-constexpr int kLocCtas = NT == kLocThreads ? 6 : NT == kLocWidest ? 1 : kKind == Loc::kOne ? 4 : 3;
+// CTAs per SM that a kernel is built for.  Blocks of some 900 tokens and more
+// (55 KB of workspace) leave room for four CTAs of 256 threads: at 61 registers
+// (64 in a batch) they fit (200 MiB text: three 423 us, four 357).  Where the
+// workspace leaves room for three, the registers of three are better (a batch of
+// 96 small files with the workspace of all kinds: 646 us, 657 built for four).
+template <int NT>
+constexpr int kLocCtas = NT == kLocThreads ? 6 : NT == kLocWide ? 4 : 1;
 
-template <int NT, Loc kKind>
-__global__ void __launch_bounds__(NT, kLocCtas<NT, kKind>) k_local(JobDev job) {
+template <int NT, Loc kKind, int kCtas>
+__global__ void __launch_bounds__(NT, kCtas) k_local(JobDev job) {
     extern __shared__ __align__(128) uint8_t sm[];
     grid_dependency_wait();  // the entropy stage's streams
     local_worker<NT, kKind>(job, sm, 0, threadIdx.x);
@@ -683,6 +684,9 @@ size_t local_smem_bytes(uint32_t T, uint32_t LB, uint32_t LIT, bool need, bool l
     return loc_layout(T, LB, LIT, need, lvl).total;
 }
 
+// CTAs of smem bytes of workspace that an SM's shared memory holds.
+static int local_fit(size_t smem) { return (int)(227 * 1024 / (smem + 1024)); }
+
 // Threads of a local CTA for a job of n_items blocks of up to T tokens whose
 // workspace has `smem` bytes.  A CTA's shared memory sets how many fit an SM:
 // with four or fewer (blocks of some 900 tokens and more), 128 threads leave
@@ -694,24 +698,36 @@ size_t local_smem_bytes(uint32_t T, uint32_t LB, uint32_t LIT, bool need, bool l
 // 256, 512 threads; one 10 KB text block 62 -> 43 -> 35).
 static int local_threads(size_t smem, uint32_t n_items, uint32_t T) {
     if (n_items <= 2u * (uint32_t)noted_sm_count()) return T > 256 ? kLocWidest : kLocWide;
-    return 227 * 1024 / (smem + 1024) <= 4 ? kLocWide : kLocThreads;
+    return local_fit(smem) <= 4 ? kLocWide : kLocThreads;
 }
 
-template <int NT, Loc kKind>
+bool local_narrow(size_t smem) { return local_threads(smem, 0xffffffffu, 0) == kLocThreads; }
+
+template <int NT, Loc kKind, int kCtas>
 static cudaError_t local_attrs(size_t smem) {
-    cudaError_t e = cudaFuncSetAttribute(k_local<NT, kKind>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_local<NT, kKind, kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess)  // the whole unified L1 as shared memory: CTAs per SM are set by their workspaces
-        e = cudaFuncSetAttribute(k_local<NT, kKind>, cudaFuncAttributePreferredSharedMemoryCarveout,
+        e = cudaFuncSetAttribute(k_local<NT, kKind, kCtas>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  cudaSharedmemCarveoutMaxShared);
     return e;
 }
 
+template <int NT, Loc kKind, int kCtas>
+static cudaError_t launch_local_ctas(const JobDev& job, int grid, size_t smem, cudaStream_t st) {
+    const cudaError_t e = local_attrs<NT, kKind, kCtas>(smem);
+    if (e != cudaSuccess) return e;
+    return launch_dependent(k_local<NT, kKind, kCtas>, grid, NT, smem, st, job);
+}
 template <int NT, Loc kKind>
 static cudaError_t launch_local_kind(const JobDev& job, int grid, size_t smem, cudaStream_t st) {
-    const cudaError_t e = local_attrs<NT, kKind>(smem);
-    if (e != cudaSuccess) return e;
-    return launch_dependent(k_local<NT, kKind>, grid, NT, smem, st, job);
+    if constexpr (NT == kLocWide) {
+        if (kKind == Loc::kAny || local_fit(smem) < kLocCtas<NT>)
+            return launch_local_ctas<NT, kKind, 3>(job, grid, smem, st);
+    }
+    if constexpr (NT != kLocWide || kKind != Loc::kAny)
+        return launch_local_ctas<NT, kKind, kLocCtas<NT>>(job, grid, smem, st);
 }
+
 template <int NT>
 static cudaError_t launch_local_nt(const JobDev& job, int grid, size_t smem, cudaStream_t st) {
     // (a batch's archives have no item tables)
@@ -720,13 +736,19 @@ static cudaError_t launch_local_nt(const JobDev& job, int grid, size_t smem, cud
     return launch_local_kind<NT, Loc::kAny>(job, grid, smem, st);
 }
 
-cudaError_t launch_local(const JobDev& job, int grid, cudaStream_t st) {
+cudaError_t launch_local(const JobDev& job_in, int grid, cudaStream_t st) {
+    JobDev job = job_in;
+    if (job.loc_hi == 0) {  // one pass over all items
+        job.loc_hi = job.n_items;
+        job.loc_ctr = 1;
+    }
     const size_t sm = local_smem_bytes(job.max_tok, job.max_lenb, job.max_lit, (job.flags & kJobNeed) != 0,
                                        (job.flags & kJobLevels) != 0);
     // a small job (a seek, a serving tick) needs no more CTAs than ticket runs
-    const uint64_t runs = (job.n_items + (uint64_t)(job.chunk ? job.chunk : 1) - 1) / (job.chunk ? job.chunk : 1);
+    const uint32_t items = job.loc_hi - job.loc_lo;
+    const uint64_t runs = (items + (uint64_t)(job.chunk ? job.chunk : 1) - 1) / (job.chunk ? job.chunk : 1);
     grid = job_grid(grid, runs);
-    const int nt = local_threads(sm, job.n_items, job.max_tok);
+    const int nt = local_threads(sm, items, job.max_tok);
     return nt == kLocWidest ? launch_local_nt<kLocWidest>(job, grid, sm, st)
            : nt == kLocWide ? launch_local_nt<kLocWide>(job, grid, sm, st)
                             : launch_local_nt<kLocThreads>(job, grid, sm, st);
@@ -795,8 +817,8 @@ cudaError_t launch_external(const JobDev& job, int grid, cudaStream_t st) {
 template <int NT>
 static int local_occupancy_nt(size_t smem) {  // (of the kind that runs most CTAs: a grid may exceed what is resident)
     int n = 0;
-    if (local_attrs<NT, Loc::kOne>(smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_local<NT, Loc::kOne>, NT, smem) != cudaSuccess)
+    if (local_attrs<NT, Loc::kOne, kLocCtas<NT>>(smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_local<NT, Loc::kOne, kLocCtas<NT>>, NT, smem) != cudaSuccess)
         return 0;
     return n;
 }

@@ -29,6 +29,7 @@ struct aceapex_batch {
     DevBuf scratch;             // streams | npend | pmap | spans | lists | job table | counters | status words
     int* d_errs = nullptr;      // [0..3] job status, [4 + a] archive a
     std::vector<int> h_errs;
+    std::vector<int> pos;       // archive -> its place in the job table
     cudaStream_t cap = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -51,6 +52,26 @@ void batch_free(aceapex_batch* B) {
     delete B;
 }
 
+// The batch's grids under parameters p, and its classes' when it has two.
+int batch_plan(aceapex_ctx* c, const aceapex_dec_params& p, const JobDev& job, LaunchPlan* lp) {
+    int rc = launch_plan(c, p, job.max_tok, job.max_lenb, job.max_lit, lp);
+    for (int k = 0; k < 2 && rc == ACEAPEX_OK && job.cls[0].items; k++) {
+        LaunchPlan t;
+        const JobDev::LocClass& C = job.cls[k];
+        rc = launch_plan(c, p, C.max_tok, C.max_lenb, C.max_lit, &t);
+        lp->grid_cls[k] = t.grid_local;
+    }
+    return rc;
+}
+
+// A batch's archives in two classes by their workspaces: run together, DNA-like
+// archives (37 KB, six CTAs of 128 threads per SM) take the workspace of text (61
+// KB for both kinds' largest streams, three CTAs of 256).  Each class gets a local
+// pass of its own when it has this many blocks per SM (96 files of up to 64 MiB,
+// 180 per SM: 1.68 -> 1.33 ms, the batch 4.63 -> 4.23); with 20 (96 files of up to 4
+// MiB) the second launch's tail takes back what it gives (647 -> 650 us).
+constexpr uint32_t kClassBlocks = 32;
+
 }  // namespace
 
 extern "C" {
@@ -71,7 +92,8 @@ int aceapex_batch_create(aceapex_ctx* c, const aceapex_batch_item* items, int n,
     std::vector<ArcJob> tab(std::max(n, 1));
     std::vector<uint64_t> o_str(n), o_np(n), o_pm(n), o_sp(n);
     uint64_t s_str = 0, s_np = 0, s_pm = 0, s_sp = 0, slots = 0, items_total = 0;
-    uint32_t max_tok = 0, max_lenb = 0, max_lit = 0;
+    JobDev::LocClass cls[2] = {};
+    std::vector<uint8_t> wide(n);
     for (int a = 0; a < n; a++) {
         const aceapex_archive* A = items[a].arc;
         if (!A || (!items[a].d_out && A->plan.total)) {
@@ -97,9 +119,12 @@ int aceapex_batch_create(aceapex_ctx* c, const aceapex_batch_item* items, int n,
         s_sp += P.span_slots * sizeof(SpanRec);
         slots += P.span_slots;
         items_total += P.n_blocks;
-        max_tok = std::max(max_tok, P.max_tok);
-        max_lenb = std::max(max_lenb, P.max_lenb);
-        max_lit = std::max(max_lit, P.max_lit);
+        wide[a] = !local_narrow(local_smem_bytes(P.max_tok, P.max_lenb, P.max_lit));
+        JobDev::LocClass& C = cls[wide[a]];
+        C.items += P.n_blocks;
+        C.max_tok = std::max(C.max_tok, P.max_tok);
+        C.max_lenb = std::max(C.max_lenb, P.max_lenb);
+        C.max_lit = std::max(C.max_lit, P.max_lit);
         B->bytes += P.total;
     }
     if (items_total >= 0xffffffffull) {
@@ -107,7 +132,15 @@ int aceapex_batch_create(aceapex_ctx* c, const aceapex_batch_item* items, int n,
         return fail(c, ACEAPEX_E_ARG, "batch_create: too many blocks in one batch");
     }
     B->blocks = items_total;
-    int rc = launch_plan(c, c->params, max_tok, max_lenb, max_lit, &B->lp);
+    JobDev& job = B->job;
+    job.max_tok = std::max(cls[0].max_tok, cls[1].max_tok);
+    job.max_lenb = std::max(cls[0].max_lenb, cls[1].max_lenb);
+    job.max_lit = std::max(cls[0].max_lit, cls[1].max_lit);
+    const uint32_t least = kClassBlocks * (uint32_t)c->n_sms;
+    const bool split = cls[0].items >= least && cls[1].items >= least &&
+                       local_narrow(local_smem_bytes(cls[0].max_tok, cls[0].max_lenb, cls[0].max_lit));
+    if (split) memcpy(job.cls, cls, sizeof cls);
+    int rc = batch_plan(c, c->params, job, &B->lp);
     if (rc) {
         batch_free(B);
         return rc;
@@ -130,10 +163,18 @@ int aceapex_batch_create(aceapex_ctx* c, const aceapex_batch_item* items, int n,
     }
     uint8_t* base = (uint8_t*)B->scratch.p;
     uint32_t item_base = 0;
-    for (int a = 0; a < n; a++) {
+    // (the job table keeps the archives' order, in two classes the narrow ones first)
+    B->pos.resize(n);
+    std::vector<int> at;
+    for (int k = 0; k < 2; k++)
+        for (int a = 0; a < n; a++)
+            if (split ? wide[a] == k : k == 0) at.push_back(a);
+    for (int t = 0; t < n; t++) {
+        const int a = at[t];
+        B->pos[a] = t;
         const aceapex_archive* A = items[a].arc;
         const Plan& P = A->plan;
-        ArcJob& J = tab[a];
+        ArcJob& J = tab[t];
         memset(&J, 0, sizeof J);
         J.arc = (const uint8_t*)A->d_arc;
         J.blk = A->d_blk;
@@ -153,7 +194,6 @@ int aceapex_batch_create(aceapex_ctx* c, const aceapex_batch_item* items, int n,
         J.order = A->d_order;
         item_base += P.n_blocks;
     }
-    JobDev& job = B->job;
     job.arcs = (const ArcJob*)(base + r_tab);
     job.n_arcs = (uint32_t)n;
     job.n_items = item_base;
@@ -162,9 +202,6 @@ int aceapex_batch_create(aceapex_ctx* c, const aceapex_batch_item* items, int n,
     job.err = B->d_errs;
     job.arc_err = B->d_errs + 4;
     job.timeout_ns = (uint64_t)c->params.timeout_us * 1000ull;
-    job.max_tok = max_tok;
-    job.max_lenb = max_lenb;
-    job.max_lit = max_lit;
     job.lists[0] = (JobDev::ListEnt*)(base + r_ls);
     job.lists[1] = job.lists[0] + slots;
     B->h_errs.assign(4 + n, 0);
@@ -177,7 +214,7 @@ int aceapex_batch_create(aceapex_ctx* c, const aceapex_batch_item* items, int n,
         return cuda_fail(c, e, "batch_create");
     }
     if ((flags & ACEAPEX_BATCH_GRAPH) && job.n_items > 0) {
-        // capture the four launches once; runs replay the graph
+        // capture the launches once; runs replay the graph
         e = cudaStreamCreateWithFlags(&B->cap, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaStreamBeginCapture(B->cap, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) {
@@ -242,7 +279,7 @@ int aceapex_batch_wait(aceapex_batch* B, void* stream, aceapex_batch_item* items
     if (items)
         for (int a = 0; a < B->n; a++)
             // an error that no archive claims (a grid-wide wait) applies to all
-            items[a].status = B->h_errs[4 + a] ? B->h_errs[4 + a] : (attributed ? ACEAPEX_OK : job_rc);
+            items[a].status = B->h_errs[4 + B->pos[a]] ? B->h_errs[4 + B->pos[a]] : (attributed ? ACEAPEX_OK : job_rc);
     if (stats) {
         memset(stats, 0, sizeof *stats);
         float t = 0;
@@ -310,8 +347,14 @@ extern "C" int aceapex_autotune(aceapex_ctx* c, const aceapex_batch_item* items,
         if (flush) cudaFree(flush);
         return cuda_fail(c, e, "autotune");
     }
-    const size_t lsm = local_smem_bytes(B->job.max_tok, B->job.max_lenb, B->job.max_lit);
-    const int occ_local = base.variant == ACEAPEX_VARIANT_PLAIN ? 1 : std::max(1, local_occupancy(lsm));
+    int occ_local = 1;
+    if (base.variant != ACEAPEX_VARIANT_PLAIN) {
+        const JobDev& j = B->job;
+        occ_local = std::max(occ_local, local_occupancy(local_smem_bytes(j.max_tok, j.max_lenb, j.max_lit)));
+        for (const JobDev::LocClass& C : j.cls)
+            if (C.items)
+                occ_local = std::max(occ_local, local_occupancy(local_smem_bytes(C.max_tok, C.max_lenb, C.max_lit)));
+    }
     std::vector<uint32_t> locals, ranss;
     for (int v : {1, 2, 3, 4, 6, 8, 12, 16})
         if (v <= occ_local) locals.push_back((uint32_t)v);
@@ -329,7 +372,7 @@ extern "C" int aceapex_autotune(aceapex_ctx* c, const aceapex_batch_item* items,
                 p.rans_ctas_per_sm = rcn;
                 p.queue_chunk = ch;
                 LaunchPlan lp;
-                if ((rc = launch_plan(c, p, B->job.max_tok, B->job.max_lenb, B->job.max_lit, &lp))) break;
+                if ((rc = batch_plan(c, p, B->job, &lp))) break;
                 B->lp = lp;
                 t.clear();
                 for (int r = 0; r <= reps && rc == ACEAPEX_OK; r++) {

@@ -116,6 +116,7 @@ std::string device_error_text(const int h[3]);
 struct LaunchPlan {
     uint32_t variant = 0, chunk = 1, wait_ns = 0;
     int grid_rans = 0, grid_local = 0, grid_plain = 0, grid_ext = 0;
+    int grid_cls[2] = {0, 0};              // a batch in two classes: the local pass's grids
     int fused_groups = 0, grid_fused = 0;  // fused entropy + local pass (whole single-archive jobs), 0: staged
 };
 // Grids for a job whose largest block has max_tok tokens, max_lenb length

@@ -138,7 +138,7 @@ struct JobDev {
     const ArcJob* arcs;       // device array of archives (batched jobs), or nullptr
     uint32_t n_arcs;
     uint32_t n_items;         // total blocks over all archives
-    uint32_t* counters;       // [1] local ticket, [2] external ticket, [3 + a] rANS ticket of archive a,
+    uint32_t* counters;       // [0], [1] local tickets, [2] external ticket, [3 + a] rANS ticket of archive a,
                               // [kStatPending] pending spans, [kStatPolls] empty cross-block polls
     int* err;                 // first error status (0 = ok)
     int* arc_err;             // per archive: first error status of that archive (batched jobs), or nullptr
@@ -146,6 +146,14 @@ struct JobDev {
     uint32_t max_tok;         // shared-memory sizing of the assembly kernel
     uint32_t max_lenb;
     uint32_t max_lit;
+    // A batch whose archives differ much in their workspaces: the items of the
+    // narrow archives come first and get a local pass of their own (host side;
+    // cls[0].items = 0: one pass over all).
+    struct LocClass {
+        uint32_t items, max_tok, max_lenb, max_lit;
+    } cls[2];
+    uint32_t loc_lo, loc_hi;  // a batch's local pass (set at its launch): items [loc_lo, loc_hi),
+    uint32_t loc_ctr;         // tickets from counters[loc_ctr]
     uint32_t flags;           // kJob* bits
     uint32_t rans_parts;      // tickets per work item of the entropy stage (set at its launch)
     uint32_t chunk;           // work items per ticket of the entropy stage and the local pass (0 = 1)

@@ -63,6 +63,8 @@ int job_grid(int full, uint64_t need);
 void note_sm_count(int n_sms);
 int noted_sm_count();
 int local_occupancy(size_t smem);
+// Does a job of many blocks run the local pass with its narrow CTAs?
+bool local_narrow(size_t smem);
 int external_occupancy();
 int plain_occupancy();
 // Copy regions out of block slots (block a at out + slot[a]*kBlock): the one

@@ -367,6 +367,14 @@ struct LocJob {
     static constexpr bool kWhole = kKind != Loc::kAny;
     static __device__ __forceinline__ bool flag(const JobDev& job, uint32_t f) { return !kWhole && (job.flags & f); }
     static __device__ __forceinline__ bool fused(const JobDev& job) { return !kWhole && job.ready; }
+    // the pass's items [first, end) and its tickets
+    static __device__ __forceinline__ uint32_t first(const JobDev& job) { return kKind == Loc::kBatch ? job.loc_lo : 0u; }
+    static __device__ __forceinline__ uint32_t end(const JobDev& job) {
+        return kKind == Loc::kBatch ? job.loc_hi : job.n_items;
+    }
+    static __device__ __forceinline__ uint32_t* tickets(const JobDev& job) {
+        return job.counters + (kKind == Loc::kBatch ? job.loc_ctr : 1u);
+    }
     static __device__ __forceinline__ int arc(const JobDev& job, uint32_t item) {
         return kKind == Loc::kOne ? 0 : find_arc(job, item);
     }
@@ -471,19 +479,19 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             pf_item = 0xffffffffu;
         } else {
             if (cleft == 0) {
-                if (tid == 0) misc[0] = atomicAdd(&job.counters[1], chunk);
+                if (tid == 0) misc[0] = atomicAdd(Kind::tickets(job), chunk);
                 grp_sync<NT>(bid);
                 cnext = misc[0];
                 cleft = chunk;
             }
-            item = Kind::kWhole ? cnext++ : ticket_item(job, cnext++);
+            item = Kind::kWhole ? Kind::first(job) + cnext++ : ticket_item(job, cnext++);
             cleft--;
         }
         // the next block's ticket: its atomic goes out now and is read at the
         // prefetch point, so its latency hides behind this block's work
         uint32_t pre_claim = 0;
         bool claimed = cleft == 0;  // group-uniform
-        if (claimed && tid == 0) pre_claim = atomicAdd(&job.counters[1], chunk);
+        if (claimed && tid == 0) pre_claim = atomicAdd(Kind::tickets(job), chunk);
         // a block that ends before the prefetch point (corrupt, or a parse-only
         // job) hands the claimed tickets on to the next iteration
         auto settle_claim = [&]() {
@@ -494,7 +502,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             cleft = chunk;
             claimed = false;
         };
-        if (item >= job.n_items) return;
+        if (item >= Kind::end(job)) return;
         const int a = Kind::arc(job, item);
         const ArcJob J = Kind::load(job, a);
         const ItemRef ir = Kind::ref(J, item - J.item_base);
@@ -747,14 +755,14 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             // ---- the stream buffers are free from here on: start the next item's
             //      copies, so that they land while this block finishes ----
             settle_claim();
-            pf_item = Kind::kWhole ? cnext++ : ticket_item(job, cnext++);
+            pf_item = Kind::kWhole ? Kind::first(job) + cnext++ : ticket_item(job, cnext++);
             cleft--;
             // (issued by the last warp, which takes the fewest in-block matches
             // below, so that its loads of the next block's descriptor delay the
             // rounds least)
             if (tid == NT - 32) {
                 // in a fused decode, only streams that are already published
-                const bool go = pf_item < job.n_items && (!Kind::fused(job) || ld_acquire_u32(job.ready + pf_item) != 0);
+                const bool go = pf_item < Kind::end(job) && (!Kind::fused(job) || ld_acquire_u32(job.ready + pf_item) != 0);
                 if (go) {
                     if (Kind::fused(job)) asm volatile("fence.proxy.async.global;" ::: "memory");
                     stage_streams<kKind>(job, pf_item, tcmd, lenb, soff, slit, tlvl, bar);
