@@ -1028,12 +1028,12 @@ def kernel_source_key():
 # other kernels.
 _GENOME = "chr1-shaped synthetic genome 253,935,557 B"
 CAPTURED_DRAM = {
-    ("98fdae1c5dff3c38", _GENOME, "k_rans"): 93797632 + 227070208,
-    ("98fdae1c5dff3c38", _GENOME, "k_local"): 223956992 + 246156288,
-    ("98fdae1c5dff3c38", _GENOME, "k_external"): 140977664 + 39984640,
+    ("89d811349d1e56f3", _GENOME, "k_rans"): 71696640 + 192153856,
+    ("89d811349d1e56f3", _GENOME, "k_local"): 223918592 + 246308352,
+    ("89d811349d1e56f3", _GENOME, "k_external"): 141579008 + 41805056,
 }
 CAPTURED_RANS_INSTR_PER_SYMBOL = {
-    ("98fdae1c5dff3c38", _GENOME): 195824333 / 221024708,
+    ("89d811349d1e56f3", _GENOME): 204397051 / 221024708,
 }
 ISSUE_PEAK = 152 * 4 * 2.07e9  # warp-instructions per second: 4 schedulers x 152 SMs x 2070 MHz
 
