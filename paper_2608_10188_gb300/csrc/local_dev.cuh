@@ -431,6 +431,16 @@ __device__ __forceinline__ bool wait_ready(const uint32_t* ready, uint32_t item,
     return true;
 }
 
+// Words of a group's `misc`: 0 its claimed ticket, 2 whether the next block's
+// streams are in flight, 3 the listed in-block matches, and one for each check
+// of a block that threads make on their own.  A check's word is cleared when
+// the block starts, set before the barrier that ends the check and read behind
+// it, and no later phase writes it: every thread reads the same verdict, however
+// late it leaves the barrier.  (`bad` decides which barriers a thread meets.
+// With one word for all checks, a warp that read a verdict late could see the
+// next check's, and run one barrier ahead of its group from there on.)
+enum : uint32_t { kChkLen = 4, kChkValue, kChkToken, kChkSource, kChkHistory, kChkDeps, kChkEnd };
+
 // The local pass of one group of NT threads (k_local: a whole CTA; k_fused: a
 // group of a fused CTA) over the job's tickets, with its workspace at sm and
 // named barrier bid; tid is the thread's index in its group.
@@ -522,7 +532,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
         if (!bad && tid == 0 && !prefetched && (!Kind::fused(job) || wait_ready(job.ready, item, deadline)))
             stage_streams<kKind>(job, item, tcmd, lenb, soff, slit, tlvl, bar);
         for (uint32_t i = tid; i < kBlock / 128; i += NT) reinterpret_cast<uint4*>(pend)[i] = make_uint4(0, 0, 0, 0);
-        if (tid == 0) misc[1] = 0;
+        if (tid < (int)(kChkEnd - kChkLen)) misc[kChkLen + tid] = 0;
         // wanted bytes of this item (all when it names none)
         const bool partial = Kind::flag(job, kJobNeed) && ir.need_n != 0;
         if (partial) {
@@ -563,11 +573,11 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                     // a value has at most three bytes
                     if (by >= 0x80 && j >= 2 && lenb[j - 1] >= 0x80 && lenb[j - 2] >= 0x80) vbad = true;
                 });
-            if (vbad) misc[1] = 1;
+            if (vbad) misc[kChkLen] = 1;
             v1[0] = c;
             block_scan<NT, 1>(v1, tot1, scanbuf, bid, tid);
         }
-        mark(tot1[0] != 2 * n || (LB > 0 && lenb[LB - 1] >= 0x80) || (LB == 0 && n > 0) || misc[1], kStageVarint);
+        mark(tot1[0] != 2 * n || (LB > 0 && lenb[LB - 1] >= 0x80) || (LB == 0 && n > 0) || misc[kChkLen], kStageVarint);
         if (!bad) {
             uint32_t idx = v1[0];
             each<kRolled>(j0, j1, 1, [&](uint32_t j) {
@@ -578,14 +588,14 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                     val = (val << 7) | (lenb[j - 1] & 0x7f);
                     if (j >= 2 && lenb[j - 2] >= 0x80) val = (val << 7) | (lenb[j - 2] & 0x7f);
                 }
-                if (val > kBlock) misc[1] = 1;
+                if (val > kBlock) misc[kChkValue] = 1;
                 const uint32_t tk = idx >> 1;
                 if (idx & 1) tml[tk] = (uint16_t)min(val, kBlock); else tll[tk] = (uint16_t)min(val, kBlock);
                 idx++;
             });
         }
         grp_sync<NT>(bid);
-        mark(misc[1] != 0, kStageVarint);
+        mark(misc[kChkValue] != 0, kStageVarint);
 
         // ---- token scans: positions, literal positions, NEW indices ----
         const uint32_t tper = (n + NT - 1) / NT;
@@ -605,11 +615,11 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                     else if (ml < J.min_match) tbad = true;
                     any_rep |= c >= 1 && c <= 4;
                 });
-            if (tbad) misc[1] = 1;
+            if (tbad) misc[kChkToken] = 1;
             v3[0] = s_len; v3[1] = s_ll; v3[2] = s_new;
             block_scan<NT, 3>(v3, tot3, scanbuf, bid, tid);
         }
-        mark(tot3[0] != R || tot3[1] != n_lit || tot3[2] != n_new || misc[1], kStageTokens);
+        mark(tot3[0] != R || tot3[1] != n_lit || tot3[2] != n_new || misc[kChkToken], kStageTokens);
         if (!bad) {
             uint32_t pos = v3[0], lp = v3[1], ni = v3[2];
             each<kRolled>(i0, i1, 1, [&](uint32_t i) {
@@ -621,7 +631,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
 #pragma unroll
                     for (int p = 0; p < 5; p++) src |= (uint64_t)soff[p * n_new + ni] << (8 * p);
                     ni++;
-                    if (src >= B + pos + ll) misc[1] = 1;  // every absolute offset precedes its destination
+                    if (src >= B + pos + ll) misc[kChkSource] = 1;  // every absolute offset precedes its destination
                 }
                 tsrc[i] = src;
                 pos += ll + ml;
@@ -629,7 +639,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
             });
         }
         any_rep = grp_or<NT>(bid, any_rep && !bad);
-        mark(misc[1] != 0, kStageSources);
+        mark(misc[kChkSource] != 0, kStageSources);
 
         // ---- the four-entry history (blocks with repeat codes only) as a
         //      warp-level scan of packed maps by warp 0, while the other warps
@@ -667,7 +677,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                     } else if (c >= 1 && c <= 4) {
                         const uint32_t j = c - 1u;
                         const uint64_t d = j == 0 ? h0 : j == 1 ? h1 : j == 2 ? h2 : h3;
-                        if (d < 1 || d > dst) misc[1] = 1;
+                        if (d < 1 || d > dst) misc[kChkHistory] = 1;
                         tsrc[i] = dst - d;
                         h3 = j >= 3 ? h2 : h3;
                         h2 = j >= 2 ? h1 : h2;
@@ -693,7 +703,7 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                     if (tll[i] > kLaneBytes) copy_run8<kRolled>(sout, slit, tlit[i], tpos[i], tll[i], lane & 7);
             }
             grp_sync<NT>(bid);
-            mark(misc[1] != 0, kStageSources);
+            mark(misc[kChkHistory] != 0, kStageSources);
         }
 
         // ---- with dependency lists: every block a match reads outside its own
@@ -710,9 +720,9 @@ __device__ __forceinline__ void local_worker(const JobDev& job, uint8_t* sm, uin
                 for (uint64_t a = tsrc[i] >> 14; a <= (e - 1) >> 14 && a < b && !dbad; a++)
                     dbad = !listed(dl, nd, (uint32_t)a);
             }
-            if (dbad) misc[1] = 1;
+            if (dbad) misc[kChkDeps] = 1;
             grp_sync<NT>(bid);
-            mark(misc[1] != 0, kStageSources);
+            mark(misc[kChkDeps] != 0, kStageSources);
         }
 
         if (Kind::flag(job, kJobIndex)) {
