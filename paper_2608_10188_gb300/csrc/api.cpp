@@ -325,7 +325,7 @@ int acx::launch_plan(aceapex_ctx* c, const aceapex_dec_params& p, uint32_t max_t
     if (lp->variant != ACEAPEX_VARIANT_PLAIN) {
         const size_t lsm =
             local_smem_bytes(max_tok, max_lenb, max_lit, (job_flags & kJobNeed) != 0, (job_flags & kJobLevels) != 0);
-        if (lsm > 227 * 1024) return fail(c, ACEAPEX_E_CORRUPT, "block too large for the local pass");
+        if (lsm > kMaxSmem) return fail(c, ACEAPEX_E_CORRUPT, "block too large for the local pass");
         if (c->occ_local_smem != lsm) {  // (an occupancy query per launch costs the serving ticks host time)
             c->occ_local = local_occupancy(lsm);
             c->occ_local_smem = lsm;

@@ -685,7 +685,7 @@ size_t local_smem_bytes(uint32_t T, uint32_t LB, uint32_t LIT, bool need, bool l
 }
 
 // CTAs of smem bytes of workspace that an SM's shared memory holds.
-static int local_fit(size_t smem) { return (int)(227 * 1024 / (smem + 1024)); }
+static int local_fit(size_t smem) { return (int)(kMaxSmem / (smem + 1024)); }
 
 // Threads of a local CTA for a job of n_items blocks of up to T tokens whose
 // workspace has `smem` bytes.  A CTA's shared memory sets how many fit an SM:
@@ -704,8 +704,8 @@ static int local_threads(size_t smem, uint32_t n_items, uint32_t T) {
 bool local_narrow(size_t smem) { return local_threads(smem, 0xffffffffu, 0) == kLocThreads; }
 
 template <int NT, Loc kKind, int kCtas>
-static cudaError_t local_attrs(size_t smem) {
-    cudaError_t e = cudaFuncSetAttribute(k_local<NT, kKind, kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+static cudaError_t local_attrs() {
+    cudaError_t e = allow_max_smem(k_local<NT, kKind, kCtas>);
     if (e == cudaSuccess)  // the whole unified L1 as shared memory: CTAs per SM are set by their workspaces
         e = cudaFuncSetAttribute(k_local<NT, kKind, kCtas>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  cudaSharedmemCarveoutMaxShared);
@@ -714,7 +714,7 @@ static cudaError_t local_attrs(size_t smem) {
 
 template <int NT, Loc kKind, int kCtas>
 static cudaError_t launch_local_ctas(const JobDev& job, int grid, size_t smem, cudaStream_t st) {
-    const cudaError_t e = local_attrs<NT, kKind, kCtas>(smem);
+    const cudaError_t e = local_attrs<NT, kKind, kCtas>();
     if (e != cudaSuccess) return e;
     return launch_dependent(k_local<NT, kKind, kCtas>, grid, NT, smem, st, job);
 }
@@ -817,7 +817,7 @@ cudaError_t launch_external(const JobDev& job, int grid, cudaStream_t st) {
 template <int NT>
 static int local_occupancy_nt(size_t smem) {  // (of the kind that runs most CTAs: a grid may exceed what is resident)
     int n = 0;
-    if (local_attrs<NT, Loc::kOne, kLocCtas<NT>>(smem) != cudaSuccess ||
+    if (local_attrs<NT, Loc::kOne, kLocCtas<NT>>() != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_local<NT, Loc::kOne, kLocCtas<NT>>, NT, smem) != cudaSuccess)
         return 0;
     return n;

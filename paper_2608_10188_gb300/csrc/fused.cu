@@ -102,13 +102,13 @@ __global__ void __launch_bounds__(kFusedMaxThreads, 1) k_fused(JobDev job, int G
 
 int fused_groups(uint32_t max_tok, uint32_t max_lenb, uint32_t max_lit, bool lvl) {
     for (int G = kFusedMaxGroups; G >= 1; G--)
-        if (fused_layout(max_tok, max_lenb, max_lit, G, lvl).total <= 227u * 1024) return G;
+        if (fused_layout(max_tok, max_lenb, max_lit, G, lvl).total <= kMaxSmem) return G;
     return 0;
 }
 
 cudaError_t launch_fused(const JobDev& job, int G, int grid, cudaStream_t st) {
     const FusedLayout F = fused_layout(job.max_tok, job.max_lenb, job.max_lit, G, (job.flags & kJobLevels) != 0);
-    cudaError_t e = cudaFuncSetAttribute(k_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F.total);
+    cudaError_t e = allow_max_smem(k_fused);
     if (e != cudaSuccess) return e;
     struct Arg {
         const JobDev* job;
@@ -134,8 +134,7 @@ cudaError_t launch_fused(const JobDev& job, int G, int grid, cudaStream_t st) {
 
 int fused_occupancy(int G, uint32_t max_tok, uint32_t max_lenb, uint32_t max_lit, bool lvl) {
     const FusedLayout F = fused_layout(max_tok, max_lenb, max_lit, G, lvl);
-    if (cudaFuncSetAttribute(k_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F.total) != cudaSuccess)
-        return 0;
+    if (allow_max_smem(k_fused) != cudaSuccess) return 0;
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused, 32 * (kFusedRansWarps + kGroupWarps * G), F.total) !=
         cudaSuccess)

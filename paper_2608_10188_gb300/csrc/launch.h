@@ -8,6 +8,17 @@
 
 namespace acx {
 
+// The most shared memory a CTA may have (sm_103a), and a kernel's permission to
+// use it.  The permission belongs to the kernel on the device, not to a launch:
+// it is always the whole, so that no thread narrows it between another's
+// permission and launch (set to each job's own workspace, 657 of 3,000 decodes of
+// two threads failed to launch).  A launch still takes what its workspace needs.
+constexpr size_t kMaxSmem = 227 * 1024;
+template <class K>
+cudaError_t allow_max_smem(K kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+}
+
 // Launch a kernel that begins with grid_dependency_wait() and may come up while
 // the kernel before it on the stream still runs (programmatic dependent launch):
 // its launch, and what it does before the wait, hide behind that kernel (10 KB

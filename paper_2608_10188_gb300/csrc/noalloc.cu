@@ -334,7 +334,7 @@ extern "C" int aceapex_decode_noalloc(const void* d_arc, uint64_t arc_len, void*
     if (out_cap < S.total) return ACEAPEX_E_ARG;
     if (S.n_blocks == 0) return ACEAPEX_OK;
     const size_t lsm = local_smem_bytes(S.max_tok, S.max_lenb, S.max_lit);
-    if (lsm > 227 * 1024) return ACEAPEX_E_CORRUPT;  // as the regular plan: no valid block needs that much
+    if (lsm > kMaxSmem) return ACEAPEX_E_CORRUPT;  // as the regular plan: no valid block needs that much
     JobDev job{};
     ArcJob& J = job.one;
     J.arc = (const uint8_t*)d_arc;
