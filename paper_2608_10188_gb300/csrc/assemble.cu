@@ -496,12 +496,10 @@ __global__ void __launch_bounds__(256) k_level_fill(JobDev job) {
 }
 
 cudaError_t launch_level_list(const JobDev& job, cudaStream_t st) {
-    k_level_scan<<<job.n_levels, kScanThreads, 0, st>>>(job);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_kernel(k_level_scan, job.n_levels, kScanThreads, 0, st, job);
     if (e != cudaSuccess) return e;
     const uint32_t grid = std::max(1u, std::min(4096u, (job.n_items + 7) / 8));
-    k_level_fill<<<grid, 256, 0, st>>>(job);
-    return cudaGetLastError();
+    return launch_kernel(k_level_fill, grid, 256, 0, st, job);
 }
 
 // Cross-block pass.  Round 0 hands the pieces out in order and a lane waits a

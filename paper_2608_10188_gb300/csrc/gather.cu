@@ -48,8 +48,7 @@ cudaError_t launch_gather(const GatherReq* one, const GatherReq* list, uint32_t 
     if (n_req == 0) return cudaSuccess;
     const uint64_t pieces = (max_len + 15) / 16;
     const uint32_t gx = (uint32_t)std::min<uint64_t>(std::max<uint64_t>((pieces + 255) / 256, 1), 1024);
-    k_gather<<<dim3(gx, n_req), 256, 0, st>>>(one ? *one : GatherReq{}, list, n_req, out, slot);
-    return cudaGetLastError();
+    return launch_kernel(k_gather, dim3(gx, n_req), 256, 0, st, one ? *one : GatherReq{}, list, n_req, out, slot);
 }
 
 }  // namespace acx

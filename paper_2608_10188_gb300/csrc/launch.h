@@ -19,6 +19,18 @@ cudaError_t allow_max_smem(K kernel) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
 }
 
+// Launch a kernel.  The status is this launch's own: reading the runtime's last
+// error behind a <<<>>> launch would report an earlier call's failure again.
+template <class K, class... A>
+cudaError_t launch_kernel(K kernel, dim3 grid, int block, size_t smem, cudaStream_t st, const A&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Launch a kernel that begins with grid_dependency_wait() and may come up while
 // the kernel before it on the stream still runs (programmatic dependent launch):
 // its launch, and what it does before the wait, hide behind that kernel (10 KB

@@ -323,8 +323,8 @@ extern "C" int aceapex_decode_noalloc(const void* d_arc, uint64_t arc_len, void*
         base = g_na_base[dev];
     }
     cudaStream_t st = (cudaStream_t)stream;
-    k_plan_small<<<1, kPlanThreads, 0, st>>>((const uint8_t*)d_arc, arc_len, base);
-    if (cudaGetLastError() != cudaSuccess) return ACEAPEX_E_CUDA;
+    if (launch_kernel(k_plan_small, 1, kPlanThreads, 0, st, (const uint8_t*)d_arc, arc_len, base) != cudaSuccess)
+        return ACEAPEX_E_CUDA;
     NaSummary S;
     if (cudaMemcpyAsync(&S, base + kOffSummary, sizeof S, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)

@@ -149,8 +149,7 @@ cudaError_t launch_plain(const JobDev& job, int grid, cudaStream_t st) {
     const size_t sm = plain_smem_bytes();
     cudaError_t e = cudaFuncSetAttribute(k_plain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_plain<<<grid, kPlainThreads, sm, st>>>(job);
-    return cudaGetLastError();
+    return launch_kernel(k_plain, grid, kPlainThreads, sm, st, job);
 }
 
 int plain_occupancy() {

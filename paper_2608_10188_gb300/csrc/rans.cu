@@ -135,8 +135,7 @@ int job_grid(int full, uint64_t need) {
 }
 
 cudaError_t launch_prologue(uint32_t* counters, uint32_t n_counters, cudaStream_t st, int* errs, uint32_t n_errs) {
-    k_prologue<<<1, 128, 0, st>>>(counters, n_counters, errs, n_errs);
-    return cudaGetLastError();
+    return launch_kernel(k_prologue, 1, 128, 0, st, counters, n_counters, errs, n_errs);
 }
 
 cudaError_t launch_rans(const JobDev& job_in, int grid, cudaStream_t st) {
