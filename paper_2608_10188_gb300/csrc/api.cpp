@@ -47,7 +47,7 @@ int aceapex_ctx_create(int device, const aceapex_dec_params* params, aceapex_ctx
     if (cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
         cudaMalloc(&c->counters, kMaxCounters * sizeof(uint32_t)) != cudaSuccess ||
         cudaMalloc(&c->d_err, 4 * sizeof(int)) != cudaSuccess ||
-        cudaMallocHost(&c->h_err, kStatusWords * sizeof(int)) != cudaSuccess ||
+        cudaMallocHost(&c->h_err, 4 * sizeof(int)) != cudaSuccess ||
         cudaMemset(c->counters, 0, kMaxCounters * sizeof(uint32_t)) != cudaSuccess ||
         cudaMemset(c->d_err, 0, 4 * sizeof(int)) != cudaSuccess) {
         aceapex_ctx_destroy(c);

@@ -28,7 +28,7 @@ struct aceapex_batch {
     LaunchPlan lp;
     DevBuf scratch;             // streams | npend | pmap | spans | lists | job table | counters | status words
     int* d_errs = nullptr;      // [0..3] job status, [4 + a] archive a
-    std::vector<int> h_errs;
+    int* h_errs = nullptr;      // pinned, the batch's own: the status words on their way back
     std::vector<int> pos;       // archive -> its place in the job table
     cudaStream_t cap = nullptr;
     cudaGraph_t graph = nullptr;
@@ -48,6 +48,7 @@ void batch_free(aceapex_batch* B) {
     if (B->cap) cudaStreamDestroy(B->cap);
     for (auto& e : B->ev)
         if (e) cudaEventDestroy(e);
+    if (B->h_errs) cudaFreeHost(B->h_errs);
     B->scratch.release();
     delete B;
 }
@@ -204,8 +205,8 @@ int aceapex_batch_create(aceapex_ctx* c, const aceapex_batch_item* items, int n,
     job.timeout_ns = (uint64_t)c->params.timeout_us * 1000ull;
     job.lists[0] = (JobDev::ListEnt*)(base + r_ls);
     job.lists[1] = job.lists[0] + slots;
-    B->h_errs.assign(4 + n, 0);
-    if (n > 0) e = cudaMemcpy(base + r_tab, tab.data(), n * sizeof(ArcJob), cudaMemcpyHostToDevice);
+    e = cudaMallocHost(&B->h_errs, (4 + (size_t)n) * sizeof(int));
+    if (e == cudaSuccess && n > 0) e = cudaMemcpy(base + r_tab, tab.data(), n * sizeof(ArcJob), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(base + r_cnt, 0, r_err - r_cnt + (4 + (uint64_t)n) * sizeof(int));
     for (auto& ev : B->ev)
         if (e == cudaSuccess) e = cudaEventCreate(&ev);
@@ -268,11 +269,10 @@ int aceapex_batch_wait(aceapex_batch* B, void* stream, aceapex_batch_item* items
     aceapex_ctx* c = B->ctx;
     cudaSetDevice(c->device);
     // the status words come back behind the work, so one wait covers both
-    cudaError_t e = cudaMemcpyAsync(c->h_err, B->d_errs, B->h_errs.size() * sizeof(int), cudaMemcpyDeviceToHost,
+    cudaError_t e = cudaMemcpyAsync(B->h_errs, B->d_errs, (4 + (size_t)B->n) * sizeof(int), cudaMemcpyDeviceToHost,
                                     (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "status words");
     if ((e = cudaStreamSynchronize((cudaStream_t)stream)) != cudaSuccess) return cuda_fail(c, e, "stream synchronize");
-    memcpy(B->h_errs.data(), c->h_err, B->h_errs.size() * sizeof(int));
     const int job_rc = B->h_errs[0];
     bool attributed = false;
     for (int a = 0; a < B->n; a++) attributed |= B->h_errs[4 + a] != 0;
@@ -302,7 +302,7 @@ int aceapex_batch_wait(aceapex_batch* B, void* stream, aceapex_batch_item* items
         stats->pending_spans = st2[kStatPending - kStatPendBytes];
         stats->wait_polls = st2[kStatPolls - kStatPendBytes];
     }
-    if (job_rc) return fail(c, job_rc, "batch: " + device_error_text(B->h_errs.data()));
+    if (job_rc) return fail(c, job_rc, "batch: " + device_error_text(B->h_errs));
     return ACEAPEX_OK;
 }
 

@@ -59,9 +59,6 @@ struct MatchIndex {
     aceapex_parse_stats stats{};  // counted from the same pass's token records
 };
 
-// Status words of a job: four, and one per archive of a batch.
-constexpr uint32_t kStatusWords = 4 + kMaxArcsPerJob;
-
 }  // namespace acx
 
 struct aceapex_ctx {
@@ -75,7 +72,7 @@ struct aceapex_ctx {
     acx::DevBuf lvl_tab, lvl_off, lvl_list;  // level-ordered decodes: per block level counts, the level list
     uint32_t* counters = nullptr;  // device
     int* d_err = nullptr;          // device
-    int* h_err = nullptr;          // pinned, kStatusWords: status words on their way back
+    int* h_err = nullptr;          // pinned: the four status words on their way back
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
     cudaStream_t s_up = nullptr, s_down = nullptr;  // decode_host: upload and download streams
     std::vector<cudaEvent_t> pipe_ev;              // decode_host: per chunk, uploaded and decoded
