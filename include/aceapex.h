@@ -105,14 +105,17 @@ typedef struct {
     uint32_t queue_chunk; /* blocks a warp (entropy stage) or CTA (local pass) takes per queue ticket (0 = 1) */
     uint32_t wait_ns;     /* cross-block pass, first round: how long a match piece may wait for its sources
                              before it is left to the later, barrier-separated rounds; 0xFFFFFFFF = no limit
-                             short of timeout_us (pieces are handed out in output order, so the lowest
-                             unfinished one always has final sources and the first round finishes them all);
-                             0 = automatic: output order, no limit; any other value takes the pieces of
-                             an archive with level bodies in level order (see ignore_levels) */
+                             short of timeout_us; 0 = automatic: no limit, pieces in output order.  In output
+                             order the lowest unfinished piece always has final sources, so without a limit
+                             the first round finishes them all.  Any value but 0 takes the pieces of an
+                             archive with level bodies in level order instead (see ignore_levels) */
     uint32_t ignore_levels; /* 0: with wait_ns set, a whole-archive decode of an archive with level bodies
                                (flags bit1) takes the cross-block matches level by level (paper, "Depth Does
-                               Not Govern Latency": the waves; a piece whose hint proves too low is left to
-                               the later rounds); 1: ignore the level bodies */
+                               Not Govern Latency": the waves).  A piece whose hint proves too low waits for
+                               wait_ns and is then left to the later rounds; with 0xFFFFFFFF there are none,
+                               so the hints are trusted: wrong ones can make every lane wait for pieces that
+                               are not handed out yet, and a valid archive then returns ACEAPEX_E_TIMEOUT.
+                               1: ignore the level bodies (output order whatever wait_ns) */
 } aceapex_dec_params;
 
 /* Timing of the last call, measured with CUDA events on the call's stream
