@@ -30,13 +30,13 @@ def acx():
 
 @pytest.fixture(scope="module")
 def parts(acx):
-    """Per kind: an archive of all but 4 of the blocks that make a class (minus
-    the one block of a bad archive beside it), and archives of 3 and 4 blocks."""
+    """Per kind: an archive of all but 5 of the blocks that make a class, and
+    archives of 3 and 4 blocks (the fifth is a corrupt archive's)."""
     import torch
     n = BLOCKS_PER_SM * torch.cuda.get_device_properties(0).multi_processor_count
     out = {}
     for kind, seed in (("dna", 5), ("text", 6)):
-        for blocks in (n - 4, 3, 4):
+        for blocks in (n - 5, 3, 4):
             data = synth.corpus(kind, blocks * BLOCK - 77, seed + blocks)
             out[kind, 1 if blocks > 4 else blocks] = data, acx.encode(data, segment=4 << 20)
     return out
@@ -45,9 +45,12 @@ def parts(acx):
 @pytest.mark.parametrize("graph,chunk,small", [(False, 1, 4), (True, 1, 4), (False, 16, 4), (False, 1, 3)])
 def test_batch_of_two_workspaces(acx, parts, graph, chunk, small):
     import torch
-    bad = build_archive([[{"cmd": 6, "lits": b"ACGT", "ml": 4, "src": 0}]])  # unknown command
-    assert oracle.decode_status(bad, verify=False)[0] == oracle.E_CORRUPT
-    cases = [parts["text", small], (None, bad), parts["dna", small], parts["text", 1], parts["dna", 1], (None, bad)]
+    # an unknown command, in a block of one token (19 KB of workspace) and of 1,501 (62 KB)
+    last = [{"cmd": 6, "lits": b"ACGT", "ml": 4, "src": 0}]
+    narrow, wide = build_archive([last]), build_archive([[{"cmd": 0, "lits": b"ACGT", "ml": 4, "src": 0}] * 1500 + last])
+    for bad in (narrow, wide):
+        assert oracle.decode_status(bad, verify=False)[0] == oracle.E_CORRUPT
+    cases = [parts["text", small], (None, wide), parts["dna", small], parts["text", 1], parts["dna", 1], (None, narrow)]
     ctx = acx.Context(0, timeout_us=2_000_000)
     try:
         ctx.set_params(queue_chunk=chunk, timeout_us=2_000_000)

@@ -146,7 +146,7 @@ def test_level_rounds_with_true_and_wrong_hints(acx, dna4m, text4m, kind):
     hints = {"true": lambda lv, b: lv, "lowered": lambda lv, b: np.maximum(lv.astype(int) - 1, 0),
              "zero": lambda lv, b: np.zeros_like(lv), "raised": lambda lv, b: np.minimum(lv.astype(int) + 3, 255),
              "random": lambda lv, b: rng.integers(0, 8, lv.size), "inverted": lambda lv, b: lv.max(initial=0) - lv}
-    # an explicit round-0 wait: level order whatever the pieces per lane
+    # an explicit round-0 wait: level order
     ctx = acx.Context(0, timeout_us=2_000_000, ctas_per_sm=1, wait_ns=20_000)
     try:
         for name, f in hints.items():
@@ -167,8 +167,8 @@ def test_level_rounds_with_true_and_wrong_hints(acx, dna4m, text4m, kind):
             assert st["pending_spans"] > 0 and st["wait_polls"] == 0, st
         finally:
             strict.close()
-        # the level bodies ignored: the round-0 hand-out
-        ctx.set_params(ignore_levels=True, timeout_us=2_000_000, ctas_per_sm=1)
+        # the level bodies ignored under the same wait: the hand-out in output order
+        ctx.set_params(ignore_levels=True, timeout_us=2_000_000, ctas_per_sm=1, wait_ns=20_000)
         rc, out = gpu_decode(ctx, arc)
         assert rc == 0 and np.array_equal(out, data)
     finally:

@@ -43,7 +43,7 @@ def test_host_pipeline_matches_oracle(acx, kind, size, kw):
     t_arc = torch.from_numpy(np.frombuffer(arc, np.uint8).copy()).pin_memory()
     t_out = torch.full((size,), 0x3C, dtype=torch.uint8).pin_memory()
     h_arc, h_out = t_arc.numpy(), t_out.numpy()
-    # a level-ordered cross-block pass whatever the pieces per lane (explicit wait)
+    # a level-ordered cross-block pass (explicit wait)
     ctx = acx.Context(0, wait_ns=20_000 if kw.get("levels") else 0)
     try:
         d_arc = torch.from_numpy(h_arc.copy()).cuda()

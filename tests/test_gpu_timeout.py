@@ -44,8 +44,8 @@ def test_dependency_wait_runs_out_then_the_context_decodes(acx):
         rc, out = gpu_decode(ctx, backwards)
         assert rc == acx.lib.E_TIMEOUT, (rc, ctx.last_error())
         assert "timed out" in ctx.last_error()
-        # the same context, default limits: the misleading hints cost time only
-        ctx.set_params(timeout_us=2_000_000)
+        # the same context, pieces waiting for a while only: the misleading hints cost time
+        ctx.set_params(timeout_us=2_000_000, wait_ns=20_000)
         rc, out = gpu_decode(ctx, backwards)
         assert rc == 0, ctx.last_error()
         assert np.array_equal(out, want)
