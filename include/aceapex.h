@@ -130,7 +130,7 @@ typedef struct {
     uint64_t blocks;  /* blocks decoded */
     uint64_t bytes;   /* bytes written to the output */
     uint64_t pending_spans;  /* matches left to the cross-block pass */
-    uint64_t wait_polls;     /* cross-block rounds after the first (the dependency depth met) */
+    uint64_t wait_polls;     /* cross-block rounds after the first (0 when no piece was deferred) */
     uint64_t pending_bytes;  /* bytes of the matches left to the cross-block pass */
 } aceapex_stats;
 

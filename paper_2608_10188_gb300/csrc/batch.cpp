@@ -6,7 +6,7 @@
 // kernels take (archive, block) work items from shared tickets across all of
 // them, so archives of very different sizes and token counts share the GPU
 // without a launch per archive (Setup, Table 1: the persistent-queue decoder
-// whose time follows the token count).  With ACEAPEX_BATCH_GRAPH the four
+// whose time follows the token count).  With ACEAPEX_BATCH_GRAPH the
 // launches are captured once into a CUDA graph and every run replays it.
 #include <cuda_runtime.h>
 #include <string.h>
@@ -69,8 +69,14 @@ int batch_plan(aceapex_ctx* c, const aceapex_dec_params& p, const JobDev& job, L
 // archives (37 KB, six CTAs of 128 threads per SM) take the workspace of text (61
 // KB for both kinds' largest streams, three CTAs of 256).  Each class gets a local
 // pass of its own when it has this many blocks per SM (96 files of up to 64 MiB,
-// 180 per SM: 1.68 -> 1.33 ms, the batch 4.63 -> 4.23); with 20 (96 files of up to 4
-// MiB) the second launch's tail takes back what it gives (647 -> 650 us).
+// 180 per SM: 1.68 -> 1.33 ms, the batch 4.63 -> 4.23).  The two passes run one
+// after the other, so in a small batch the second one's tail takes back what the
+// split gives: 96 files of mixed sizes up to 4 MiB, 20 per SM, 647 us in one pass
+// and 650 in two.  With files of one size two passes are even at 8 to 16 and
+// ahead from there (96 files, 8 / 12 / 16 / 20 / 32 / 64 / 96 per SM: 312 / 407 / 547
+// / 650 / 945 / 1730 / 2499 us in one, 317 / 394 / 533 / 634 / 910 / 1646 / 2388 in
+// two; 8 files, 8 / 16 / 24 / 32 / 64: 287 / 462 / 693 / 852 / 1577 and 292 / 460 / 673
+// / 818 / 1508).  The line lies where every mix measured gains.
 constexpr uint32_t kClassBlocks = 32;
 
 }  // namespace

@@ -83,7 +83,7 @@ struct ArcJob {
     uint8_t* scratch;         // decoded streams
     uint8_t* out;             // output: block b at out + b*kBlock
     uint32_t* npend;          // per block: number of pending spans after the local pass
-    uint32_t* pmap;           // per block pending-byte bitmap, 512 words (valid when npend > 0)
+    uint32_t* pmap;           // per block pending-byte bitmap, 512 words (written for every block)
     SpanRec* spans;           // pending pieces, slots [span_base, span_base + n_tok + kSpanSlack) per block
     uint64_t total;           // decompressed size
     uint32_t n_blocks;

@@ -182,13 +182,11 @@ __device__ __forceinline__ void pend_update_smem(uint32_t* pend, uint32_t s, uin
     });
 }
 
-// Run copy out[b, b+L) = src[a, a+L) (both in shared memory, the two ranges
-// disjoint: a literal run, or an in-block match at distance >= L), by the
-// eight lanes sl = 0..7 of a lane group: 16-byte stores in the middle, each
-// from five funnel-shifted source words, bytes at the ragged ends.  Source
-// words may reach 3 bytes past the run, still inside the buffer (the literal
-// buffer is padded; a match source ends at or before its destination, which
-// holds at least 4 bytes); those bytes are shifted out unused.
+// Literal run out[b, b+L) = lit[a, a+L) (both in shared memory), by the eight
+// lanes sl = 0..7 of a lane group: 16-byte stores in the middle, each from five
+// funnel-shifted source words, bytes at the ragged ends.  Source words may reach
+// 4 bytes past the run (the fifth of an aligned one), inside the literal buffer's
+// 16 bytes of padding; those bytes are not used.
 template <bool kRolled>
 __device__ __forceinline__ void copy_run8(uint8_t* sout, const uint8_t* lit, uint32_t a, uint32_t b, uint32_t L,
                                           uint32_t sl) {
@@ -213,8 +211,9 @@ __device__ __forceinline__ void copy_run8(uint8_t* sout, const uint8_t* lit, uin
 
 // Copy out[o, o + ml) = out[so, so + ml) (disjoint), by one thread: bytes up to
 // a word boundary of the destination, words from two source words each, four
-// at a time, bytes at the end.  Words may reach 3 bytes past the source run
-// (never past the block: a source ends at or before its destination).
+// at a time, bytes at the end.  Words may reach 4 bytes past the source run (the
+// second word of an aligned one, loaded and not used), never past the block: a
+// source ends at or before its destination, which holds at least 4 bytes.
 __device__ __forceinline__ void copy_lane(uint8_t* out, uint32_t so, uint32_t o, uint32_t ml) {
     const uint32_t e = o + ml, q0 = (o + 3) >> 2, q1 = e >> 2;
     const uint32_t head = min(4 * q0, e), tail = max(4 * q1, head);
@@ -261,8 +260,8 @@ __device__ __forceinline__ void fill_run8(uint8_t* out, uint32_t so, uint32_t o,
 // of a lane group: whole destination words from two source words each, bytes
 // at the ragged ends.  An in-block match is short (30 bytes on average in a
 // genome), where the 16-byte chunks of copy_run8 are mostly ragged ends.
-// Words may reach 3 bytes past the source run (never past the block: a source
-// ends at or before its destination).
+// Words may reach 4 bytes past the source run, never past the block (as in
+// copy_lane).
 template <bool kRolled>
 __device__ __forceinline__ void copy_words8(uint8_t* out, uint32_t so, uint32_t o, uint32_t ml, uint32_t sl) {
     const uint32_t e = o + ml, q0 = (o + 3) >> 2, q1 = e >> 2;  // whole words [q0, q1)
