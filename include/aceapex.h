@@ -25,7 +25,9 @@
  *  - Return value: ACEAPEX_OK (0) or a negative ACEAPEX_E_* status.  The
  *    library never prints; aceapex_last_error() gives a message.
  *  - "device pointer": memory of the context's CUDA device (cudaMalloc or a
- *    framework allocator); "host pointer": ordinary host memory.
+ *    framework allocator); "host pointer": ordinary host memory.  Archives that
+ *    are decoded from device memory, and whole-archive outputs of 16 bytes or
+ *    more, must be 16-byte aligned (else ACEAPEX_E_ARG); regions may go anywhere.
  *  - "stream": a cudaStream_t passed as void* (NULL = the legacy default
  *    stream).  Decode calls enqueue work on it; the synchronous variants then
  *    synchronise that stream and read the device error word.

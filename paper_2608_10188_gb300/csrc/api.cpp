@@ -246,6 +246,8 @@ static int enqueue_decode(aceapex_ctx* c, aceapex_archive* A, const void* d_arc,
                           bool timed, uint32_t lo = 0, uint32_t hi = 0xffffffffu) {
     const Plan& P = A->plan;
     if (hi > P.n_blocks) hi = P.n_blocks;
+    if (!arc_aligned(P, d_arc) || !out_aligned(P, d_out))
+        return fail(c, ACEAPEX_E_ARG, "decode: archive or output not 16-byte aligned");
     cudaError_t e;
     const size_t nb = std::max<size_t>(P.n_blocks, 1);
     if ((e = c->streams.ensure(P.scratch_bytes)) != cudaSuccess) return cuda_fail(c, e, "scratch allocation");

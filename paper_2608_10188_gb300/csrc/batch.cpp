@@ -115,6 +115,10 @@ int aceapex_batch_create(aceapex_ctx* c, const aceapex_batch_item* items, int n,
             batch_free(B);
             return fail(c, ACEAPEX_E_ARG, "batch_create: item " + std::to_string(a) + " output buffer too small");
         }
+        if (!arc_aligned(A->plan, A->d_arc) || !out_aligned(A->plan, items[a].d_out)) {
+            batch_free(B);
+            return fail(c, ACEAPEX_E_ARG, "batch_create: item " + std::to_string(a) + " archive or output not 16-byte aligned");
+        }
         const Plan& P = A->plan;
         o_str[a] = s_str;
         s_str += up(P.scratch_bytes, 256);

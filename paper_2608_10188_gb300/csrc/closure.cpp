@@ -122,6 +122,7 @@ void finish_runs(aceapex_parse_stats& S, std::vector<uint32_t>& runs) {
 int acx::build_match_index(aceapex_ctx* c, aceapex_archive* A) {
     if (A->midx) return ACEAPEX_OK;
     const Plan& P = A->plan;
+    if (!arc_aligned(P, A->d_arc)) return fail(c, ACEAPEX_E_ARG, "match index: archive not 16-byte aligned");
     MatchIndex* M = new (std::nothrow) MatchIndex();
     if (!M) return fail(c, ACEAPEX_E_NOMEM, "match index: host allocation");
     M->first.assign((size_t)P.n_blocks + 1, 0);

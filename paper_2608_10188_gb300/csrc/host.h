@@ -106,6 +106,12 @@ inline int cuda_fail(aceapex_ctx* c, cudaError_t e, const char* where) {
     return fail(c, ACEAPEX_E_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
+// The kernels read archive bytes and write blocks 16 bytes at a time: a device
+// archive with blocks, and a whole output of 16 bytes or more, must lie on a
+// 16-byte boundary (any other address would fault the device).
+inline bool arc_aligned(const Plan& P, const void* d_arc) { return P.n_blocks == 0 || ((uintptr_t)d_arc & 15) == 0; }
+inline bool out_aligned(const Plan& P, const void* d_out) { return P.total < 16 || ((uintptr_t)d_out & 15) == 0; }
+
 // Text of a device-reported error (err[0..2] as the kernels write it).
 std::string device_error_text(const int h[3]);
 

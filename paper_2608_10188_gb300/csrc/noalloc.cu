@@ -333,6 +333,8 @@ extern "C" int aceapex_decode_noalloc(const void* d_arc, uint64_t arc_len, void*
     if (S.status != 0) return ACEAPEX_E_CORRUPT;
     if (out_cap < S.total) return ACEAPEX_E_ARG;
     if (S.n_blocks == 0) return ACEAPEX_OK;
+    // the kernels move 16 bytes at a time (see the regular path's check)
+    if (((uintptr_t)d_arc & 15) || (S.total >= 16 && ((uintptr_t)d_out & 15))) return ACEAPEX_E_ARG;
     const size_t lsm = local_smem_bytes(S.max_tok, S.max_lenb, S.max_lit);
     if (lsm > kMaxSmem) return ACEAPEX_E_CORRUPT;  // as the regular plan: no valid block needs that much
     JobDev job{};

@@ -96,6 +96,7 @@ extern "C" int aceapex_decode_range(aceapex_ctx* c, aceapex_archive* A, uint64_t
     if (start > P.total || len > P.total - start) return fail(c, ACEAPEX_E_RANGE, "decode_range: range outside the archive");
     if (stats) memset(stats, 0, sizeof *stats);
     if (len == 0) return ACEAPEX_OK;
+    if (!arc_aligned(P, A->d_arc)) return fail(c, ACEAPEX_E_ARG, "decode_range: archive not 16-byte aligned");
     cudaSetDevice(c->device);
     cudaStream_t st = (cudaStream_t)stream;
     const uint32_t b0 = (uint32_t)(start / kBlock), b1 = (uint32_t)((start + len - 1) / kBlock);
