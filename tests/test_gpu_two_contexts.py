@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 
 def _archive(tokens, lits, ml):
-    arc = build_archive([[{"cmd": 0, "lits": lits, "ml": ml, "src": 0}] * tokens] * 1)
+    arc = build_archive([[{"cmd": 0, "lits": lits, "ml": ml, "src": 0}] * tokens])
     return arc, oracle.decode(arc, verify=False)
 
 
